@@ -101,8 +101,6 @@ bool refocus_supported(int ha, int wa, int hb, int wb);
 // ([planes][hb][ha][wa] floats), plus a row-padded copy of Gamma when its rows
 // do not meet the staging alignment.  0 if unsupported.
 size_t refocus_ws_bytes(int ha, int wa, int hb, int wb, int n_planes);
-// Kernel launches of one refocusing call.
-int refocus_launches(int ha, int wa, int n_planes);
 // Whole refocusing of gamma_f32 (slice-major [hb*wb][ha*wa]) into out
 // ([n_planes][ha][wa]); alpha, beta: host arrays of n_planes coefficients.
 cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, const double* alpha,
@@ -125,7 +123,6 @@ struct Refocus4dLayout {                   // byte offsets in the workspace
     size_t tables, c_hi, c_lo, bytes;
 };
 Refocus4dLayout refocus4d_layout(int ha, int wa, int hb, int wb, int n_planes);
-bool refocus4d_box_fits(int wa, int wb);
 // planes of one chunk (np <= layout.chunk); out = [np][ha][wa]
 cudaError_t launch_refocus4d_chunk(const float* gamma_f32, int ha, int wa, int hb, int wb, const Plane4Block& coef,
                                    int np, uint8_t* ws, const Refocus4dLayout& L, float* out, cudaStream_t st);
@@ -133,47 +130,45 @@ cudaError_t launch_refocus4d_chunk(const float* gamma_f32, int ha, int wa, int h
 // ------------------------------------------------------------------ denoiser
 constexpr int kDenoiserParams = 21409;    // model blob floats
 constexpr int kDenoiseParts = 456;        // CTAs of a weight-gradient pass (fixed-order partials; 3 x 152 SMs)
-struct DenoiseLayout {                    // byte offsets in the workspace
-    size_t scale, sums, x0, a1, a2, a3, y, dy, d_hi, d_lo, part;
-    // tensor-core forward (widths 32, 64, 128): channels-last copies of x (padded
-    // to 32 channels), a1 and a2, and the bf16 weights of layers 0..2; tc = 0 if
-    // the width does not allow it
-    int tc;
-    size_t xc, c1, c2, wt;
-    // tensor-core weight gradients (training, width 64): the layer's output
-    // gradient as two bf16 terms [slice][2 Cout][H][W], x-shifted copies of the
-    // layer input [slice][3 Cin'][H][W] (Cin' = 16 or 32), per-CTA partial sums
-    // and per-block bias sums; wg = 0 if the width does not allow it
-    int wg;
-    size_t dsplit, shifted, wgpart, bpart;
-    // and the input gradients of layers 2 and 1 on the tensor cores: the split
-    // delta channels-last (hi, lo) and the flipped bf16 weights of layers 1, 2
-    size_t dcl_hi, dcl_lo, wtb, bytes;
+struct DenoiseLayout {                    // byte offsets in the workspace (direct convolutions)
+    size_t scale, sums, x0, a1, a2, a3, y, dy, d_hi, d_lo, part, bytes;
 };
-constexpr int kWgMaxCtas = 152 * 2;       // CTAs of a tensor-core weight-gradient pass (partial slots)
-// Tiled tensor map over a bfloat16 array of rank 3 or 4 with 64-byte swizzle
-// (box innermost extent 64 bytes); dims innermost first, strides in bytes for
-// dims 1..rank-1.  False if the driver rejects it.
-bool make_bf16_map_sw64(CUtensorMap* m, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
-                        const uint32_t* box);
-// As make_bf16_map_sw64 with 128-byte swizzle (box innermost extent 128 bytes).
-bool make_bf16_map_sw128(CUtensorMap* m, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
-                         const uint32_t* box);
 DenoiseLayout denoise_layout(int ha, int wa, int hb, int wb, bool training);
-// scale, stacked input, activations and y of the network on gamma_in (keep_cf:
-// also the channels-first activations the backward pass reads; status,
-// timeout_ns: the bounded waits of the tensor-core layers)
+// scale, stacked input, activations and y of the network on gamma_in
 cudaError_t denoise_forward(const float* model, const float* gamma_in, int ha, int wa, int hb, int wb,
-                            uint8_t* ws, const DenoiseLayout& L, bool keep_cf, unsigned int* status,
-                            unsigned long long timeout_ns, cudaStream_t st);
+                            uint8_t* ws, const DenoiseLayout& L, cudaStream_t st);
 cudaError_t denoise_output(const uint8_t* ws, const DenoiseLayout& L, int64_t n, float* gamma_out,
                            cudaStream_t st);
 // after denoise_forward: loss and gradient of the model blob
 cudaError_t denoise_backward(const float* model, const float* gamma_target, int ha, int wa, int hb, int wb,
-                             uint8_t* ws, const DenoiseLayout& L, float* grad, float* loss, int sm_count,
-                             unsigned int* status, unsigned long long timeout_ns, cudaStream_t st);
+                             uint8_t* ws, const DenoiseLayout& L, float* grad, float* loss, cudaStream_t st);
 cudaError_t denoise_adam(float* model, float* m, float* v, const float* grad, int64_t step, float lr,
                          cudaStream_t st);
+
+// The denoiser over one padded line of pixels (denoise_line.cu), for images of any
+// width.
+constexpr int kDnSumBlocks = 256;
+constexpr int kDnMaxCtas = 152;   // CTAs of a training pass (partial sums)
+struct DnFlat {
+    int H, W, Wp;             // image, and its padded row (W + 1 or up to 3 more)
+    bool tensor;              // forward layers on the tensor cores
+    uint32_t Q;               // positions of the line: slices x (H + 1) x (W + 1)
+    int T, n_units;           // a convolution's 128-pixel tiles per unit, and its units
+    int bstride, SP;          // staged pixels between the rows' bands, staged pixels per plane
+    int64_t G, PL;            // front margin and length of a plane, in pixels
+    // byte offsets in the workspace; training: xin, act[0..2] = a1..a3, lo terms,
+    // dy records, partial sums
+    size_t scale, sums, wt, act[3], xin, lo[2], rec, part, bpart;
+};
+// False when the line's buffers do not fit ws_bytes (images of few pixels).
+bool dn_flat_plan(int ha, int wa, int hb, int wb, bool training, size_t ws_bytes, DnFlat* out);
+// loss and gradient of the model blob
+cudaError_t dn_flat_grad(const DnFlat& g, const float* model, const float* gamma_in, const float* gamma_target, int hb,
+                         int wb, uint8_t* ws, float* grad, float* loss, int sm_count, unsigned int* status,
+                         unsigned long long timeout_ns, cudaStream_t st);
+cudaError_t dn_flat_denoise(const DnFlat& g, const float* model, const float* gamma_in, float* gamma_out, int hb, int wb,
+                            uint8_t* ws, int sm_count, unsigned int* status, unsigned long long timeout_ns,
+                            cudaStream_t st);
 
 // ------------------------------------------------------------------ self test
 cudaError_t launch_wait_selftest(unsigned int* status, unsigned long long timeout_ns,
