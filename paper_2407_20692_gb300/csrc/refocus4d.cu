@@ -25,12 +25,15 @@
 //
 // This file is compiled without FMA contraction (Kahan steps).
 #include "kernels.cuh"
+#include "ptx.cuh"
 
 namespace cpi {
 namespace {
 
 constexpr int kPad = 2;              // zero border of the staged box
 constexpr int kR4Threads = 256;
+
+constexpr long long kXBias = 128ll + ((long long)kPad << 32);
 
 __device__ __forceinline__ long long r4_fix(double v) { return __double2ll_rn(v * 4294967296.0); }
 
@@ -53,6 +56,7 @@ __device__ __forceinline__ void r4_kahan(float& acc, float& cmp, float v) {
 // Per-plane coordinate tables (fixed point), chunk planes p0 .. p0 + np - 1:
 //   x axis: TAx[p][c] = alpha (c - cxa) + cxa,        TBx[p][j] = beta sx (j - cxb)
 //           TAbx[p][c] = gamma (c - cxa) / sx + cxb,  TBbx[p][j] = delta (j - cxb)
+//           (TAx and TAbx with the 24-bit rounding bias and the box's border added)
 //   y axis: the same with rows (ha, hb, sy).
 __global__ void r4_tables_kernel(const Plane4Block co, int np, int ha, int wa, int hb, int wb,
                                  long long* __restrict__ t, int64_t stride) {
@@ -70,8 +74,8 @@ __global__ void r4_tables_kernel(const Plane4Block co, int np, int ha, int wa, i
     long long* TBy = t + 6 * stride + (int64_t)p * hb;
     long long* TBby = t + 7 * stride + (int64_t)p * hb;
     for (int c = threadIdx.x; c < wa; c += blockDim.x) {
-        TAx[c] = r4_fix(al * (c - cxa) + cxa);
-        TAbx[c] = r4_fix(ga * (c - cxa) / sx + cxb);
+        TAx[c] = r4_fix(al * (c - cxa) + cxa) + kXBias;
+        TAbx[c] = r4_fix(ga * (c - cxa) / sx + cxb) + kXBias;
     }
     for (int j = threadIdx.x; j < wb; j += blockDim.x) {
         TBx[j] = r4_fix(be * sx * (j - cxb));
@@ -87,100 +91,185 @@ __global__ void r4_tables_kernel(const Plane4Block co, int np, int ha, int wa, i
     }
 }
 
-// Stage 1: CTA (yb, ya0 .. ya0 + K - 1): the K boxes of those row pairs; every
-// plane of the chunk, G planes at a time; thread w of a pass takes plane
-// p0 + w / wa and column x_c = w % wa (so narrow images still give every thread
-// work).  The taps of (plane, x_c, j_c) do not depend on the row pair, so each is
-// formed once and applied to all K boxes.  sB holds the G planes' angular-column
-// tables.
-constexpr int kColThreads = 512;
-template <bool kSmem, int K>
-__global__ void __launch_bounds__(kColThreads) r4_cols_kernel(const float* __restrict__ g, int np, int G, int ha,
-                                                              int wa, int hb, int wb, const long long* __restrict__ t,
-                                                              int64_t stride, float* __restrict__ c_hi,
-                                                              float* __restrict__ c_lo) {
+// Stage 1: CTA (yb, ya0 .. ya0 + K - 1): the boxes of those K row pairs, interleaved
+// in shared memory as [xb][xa][K rows]; every plane of the chunk, G planes at a time;
+// thread w of a pass takes plane p0 + w / wa and column x_c = w % wa (so narrow images
+// still give every thread work).  The taps of (plane, x_c, j_c) do not depend on the
+// row pair: each is formed once and one 4, 8 or 16-byte load fetches it for all K
+// rows, whose sums run in packed FP32 lanes.  About 26 instructions form the taps, 4
+// load, and 10 K / 2 sum, so K = 4 wherever the box fits, else 2 (128 x 128), else 1.
+// The pitch of the box's rows is one entry short of (or past) a whole number of bank
+// cycles: with alpha > 1 the lanes of a load spread over more than one cycle of banks,
+// and where gamma has the sign of alpha - 1 they also step to the next row as they
+// spread, so a row that starts one entry early brings them back (the other sign: one
+// entry late).  Counted over 41 planes at 128 x 128, K = 2: 10.9 wavefronts per 4
+// loads against 15.7 with rows on the same bank; 8 is the least.  sB holds
+// the G planes' angular-column tables.  Bound by the issue of the taps and by the
+// shared-memory reads (4 K bytes x 4 taps a thread).
+template <int K>
+struct BoxOf;
+template <>
+struct BoxOf<1> {
+    typedef float T;
+    static __device__ __forceinline__ void set(T& b, const float* v) { b = v[0]; }
+};
+template <>
+struct BoxOf<2> {
+    typedef f32x2 T;
+    static __device__ __forceinline__ void set(T& b, const float* v) { b = pk2(v[0], v[1]); }
+};
+template <>
+struct BoxOf<4> {
+    typedef ulonglong2 T;
+    static __device__ __forceinline__ void set(T& b, const float* v) { b = make_ulonglong2(pk2(v[0], v[1]), pk2(v[2], v[3])); }
+};
+
+__device__ __forceinline__ void r4_kahan2(f32x2& acc, f32x2& cmp, f32x2 v) {
+    const f32x2 y = sub2(v, cmp);
+    const f32x2 t = add2(acc, y);
+    cmp = sub2(sub2(t, acc), y);
+    acc = t;
+}
+// one bilinear sample of both lanes, Kahan-added
+__device__ __forceinline__ void r4_sample2(f32x2& acc, f32x2& cmp, f32x2 fa, f32x2 ga, f32x2 fb, f32x2 gb, f32x2 v00,
+                                           f32x2 v01, f32x2 v10, f32x2 v11) {
+    const f32x2 top = fma2(fa, v01, mul2(ga, v00));
+    const f32x2 bot = fma2(fa, v11, mul2(ga, v10));
+    r4_kahan2(acc, cmp, fma2(fb, bot, mul2(gb, top)));
+}
+
+constexpr int kColThreads = 1024;      // at most; 512 where two CTAs fit an SM
+template <int K>
+__global__ void __launch_bounds__(kColThreads, 1) r4_cols_kernel(const float* __restrict__ g, int np, int G, int ha,
+                                                                 int wa, int hb, int wb, int WP,
+                                                                 const long long* __restrict__ t, int64_t stride,
+                                                                 float* __restrict__ c_hi, float* __restrict__ c_lo) {
+    typedef typename BoxOf<K>::T Box;
+    constexpr int NP = K > 1 ? K / 2 : 1;                  // packed sums per thread
     extern __shared__ __align__(16) float sm[];
-    const int yb = blockIdx.x, ya0 = blockIdx.y * K;
-    const int nb = min(K, ha - ya0);                       // boxes of this CTA
+    const int yb = blockIdx.x, ya0 = blockIdx.y * K, nt = blockDim.x;
+    const int nb = min(K, ha - ya0);                       // rows of this CTA
     const int64_t ma = (int64_t)ha * wa;
-    const int WP = wa + 2 * kPad, HP = wb + 2 * kPad;     // padded box: HP rows (xb) x WP columns (xa)
-    const int BS = HP * WP;
-    long long* sB = reinterpret_cast<long long*>(sm);      // [G][2][wb]: TBx, TBbx of the pass's planes
-    float* box = reinterpret_cast<float*>(sB + 2 * (size_t)G * wb);   // [K][HP][WP]
-    if constexpr (kSmem) {
-        for (int k = 0; k < nb; ++k)
-            for (int i = threadIdx.x; i < BS; i += kColThreads) {
-                const int r = i / WP, q = i - r * WP;
-                const int xb = r - kPad, xa = q - kPad;
-                box[k * BS + i] = (xb >= 0 && xb < wb && xa >= 0 && xa < wa)
-                                      ? g[(int64_t)(yb * wb + xb) * ma + (int64_t)(ya0 + k) * wa + xa]
-                                      : 0.0f;
-            }
+    const int HP = wb + 2 * kPad;                          // padded box: HP rows (xb) x WP columns (xa)
+    longlong2* sB = reinterpret_cast<longlong2*>(sm);      // [G][wb]: (TBx, TBbx) of the pass's planes
+    Box* box = reinterpret_cast<Box*>(sB + (size_t)G * wb);
+    for (int i = threadIdx.x; i < HP * WP; i += nt) {
+        const int r = i / WP, xb = r - kPad, xa = i - r * WP - kPad;
+        float v[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            v[k] = (k < nb && xb >= 0 && xb < wb && xa >= 0 && xa < wa)
+                       ? __ldg(g + (int64_t)(yb * wb + xb) * ma + (int64_t)(ya0 + k) * wa + xa)
+                       : 0.0f;
+        BoxOf<K>::set(box[i], v);
     }
     for (int p0 = 0; p0 < np; p0 += G) {
         const int gp = min(G, np - p0);
         __syncthreads();   // boxes ready / previous pass's tables consumed
-        for (int i = threadIdx.x; i < gp * wb; i += kColThreads) {
+        for (int i = threadIdx.x; i < gp * wb; i += nt) {
             const int k = i / wb, j = i - k * wb;
-            sB[(2 * k) * wb + j] = t[2 * stride + (int64_t)(p0 + k) * wb + j];
-            sB[(2 * k + 1) * wb + j] = t[3 * stride + (int64_t)(p0 + k) * wb + j];
+            sB[i] = make_longlong2(t[2 * stride + (int64_t)(p0 + k) * wb + j], t[3 * stride + (int64_t)(p0 + k) * wb + j]);
         }
         __syncthreads();
-        for (int w = threadIdx.x; w < gp * wa; w += kColThreads) {
+        for (int w = threadIdx.x; w < gp * wa; w += nt) {
             const int kp = w / wa, xc = w - kp * wa, p = p0 + kp;
-            const long long* B = sB + 2 * kp * wb;
+            const longlong2* B = sB + kp * wb;
             const long long ax = t[0 * stride + (int64_t)p * wa + xc];
             const long long abx = t[1 * stride + (int64_t)p * wa + xc];
-            float acc[K], cmp[K];
+            f32x2 acc[NP], cmp[NP];
+            float acc1 = 0.0f, cmp1 = 0.0f;
 #pragma unroll
-            for (int k = 0; k < K; ++k) acc[k] = cmp[k] = 0.0f;
+            for (int k = 0; k < NP; ++k) acc[k] = cmp[k] = 0ull;
+#pragma unroll (K == 1 ? 4 : 2)
             for (int jc = 0; jc < wb; ++jc) {
-                const R4Frac fa = r4_split(ax + B[jc]);
-                const R4Frac fb = r4_split(abx + B[wb + jc]);
-                const float ga = 1.0f - fa.f, gb = 1.0f - fb.f;
-                if constexpr (kSmem) {
-                    const int xa = min(max(fa.i, -kPad), wa) + kPad;
-                    const int xb = min(max(fb.i, -kPad), wb) + kPad;
-                    const float* q0 = box + xb * WP + xa;
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        if (k < nb) {
-                            const float* q = q0 + k * BS;
-                            const float top = __fmaf_rn(fa.f, q[1], ga * q[0]);
-                            const float bot = __fmaf_rn(fa.f, q[WP + 1], ga * q[WP]);
-                            r4_kahan(acc[k], cmp[k], __fmaf_rn(fb.f, bot, gb * top));
-                        }
-                    }
+                const longlong2 b = B[jc];
+                const long long ua = ax + b.x, ub = abx + b.y;
+                const int xa = min(max((int)(ua >> 32), 0), wa + kPad);
+                const int xb = min(max((int)(ub >> 32), 0), wb + kPad);
+                const float fa = (float)((uint32_t)ua >> 8) * 0x1p-24f, ga = 1.0f - fa;
+                const float fb = (float)((uint32_t)ub >> 8) * 0x1p-24f, gb = 1.0f - fb;
+                const Box* q = box + xb * WP + xa;
+                if constexpr (K == 1) {
+                    const float top = __fmaf_rn(fa, q[1], ga * q[0]);
+                    const float bot = __fmaf_rn(fa, q[WP + 1], ga * q[WP]);
+                    r4_kahan(acc1, cmp1, __fmaf_rn(fb, bot, gb * top));
                 } else {
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        if (k < nb) {
-                            const float* gbase = g + ((int64_t)yb * wb) * ma + (int64_t)(ya0 + k) * wa;
-                            float s[2][2];
-#pragma unroll
-                            for (int db = 0; db < 2; ++db)
-#pragma unroll
-                                for (int da = 0; da < 2; ++da) {
-                                    const int xa = fa.i + da, xb = fb.i + db;
-                                    s[db][da] = (xa >= 0 && xa < wa && xb >= 0 && xb < wb)
-                                                    ? __ldg(gbase + (int64_t)xb * ma + xa)
-                                                    : 0.0f;
-                                }
-                            const float top = __fmaf_rn(fa.f, s[0][1], ga * s[0][0]);
-                            const float bot = __fmaf_rn(fa.f, s[1][1], ga * s[1][0]);
-                            r4_kahan(acc[k], cmp[k], __fmaf_rn(fb.f, bot, gb * top));
-                        }
+                    const f32x2 fa2 = pk2(fa, fa), ga2 = pk2(ga, ga), fb2 = pk2(fb, fb), gb2 = pk2(gb, gb);
+                    if constexpr (K == 2) {
+                        r4_sample2(acc[0], cmp[0], fa2, ga2, fb2, gb2, q[0], q[1], q[WP], q[WP + 1]);
+                    } else {
+                        const ulonglong2 v00 = q[0], v01 = q[1], v10 = q[WP], v11 = q[WP + 1];
+                        r4_sample2(acc[0], cmp[0], fa2, ga2, fb2, gb2, v00.x, v01.x, v10.x, v11.x);
+                        r4_sample2(acc[1], cmp[1], fa2, ga2, fb2, gb2, v00.y, v01.y, v10.y, v11.y);
                     }
                 }
             }
+            int64_t o = (((int64_t)p * ha + ya0) * hb + yb) * wa + xc;
+            if constexpr (K == 1) {
+                c_hi[o] = acc1;
+                c_lo[o] = -cmp1;
+            } else {
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                if (k < nb) {
-                    const int64_t o = (((int64_t)p * ha + ya0 + k) * hb + yb) * wa + xc;
-                    c_hi[o] = acc[k];
-                    c_lo[o] = -cmp[k];
+                for (int k = 0; k < K; ++k, o += (int64_t)hb * wa) {
+                    float s[2], e[2];
+                    unpk2(acc[k / 2], s[0], s[1]);
+                    unpk2(cmp[k / 2], e[0], e[1]);
+                    if (k < nb) {
+                        c_hi[o] = s[k & 1];
+                        c_lo[o] = -e[k & 1];
+                    }
                 }
             }
+        }
+    }
+}
+
+// The same for a box too large for shared memory (256 x 256): one row pair per CTA,
+// taps read from global memory.
+constexpr int kColThreadsG = 512;
+__global__ void __launch_bounds__(kColThreadsG) r4_cols_global_kernel(const float* __restrict__ g, int np, int G, int ha,
+                                                                      int wa, int hb, int wb,
+                                                                      const long long* __restrict__ t, int64_t stride,
+                                                                      float* __restrict__ c_hi, float* __restrict__ c_lo) {
+    extern __shared__ __align__(16) float sm[];
+    const int yb = blockIdx.x, ya = blockIdx.y;
+    const int64_t ma = (int64_t)ha * wa;
+    longlong2* sB = reinterpret_cast<longlong2*>(sm);
+    const float* gbase = g + ((int64_t)yb * wb) * ma + (int64_t)ya * wa;
+    for (int p0 = 0; p0 < np; p0 += G) {
+        const int gp = min(G, np - p0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < gp * wb; i += kColThreadsG) {
+            const int k = i / wb, j = i - k * wb;
+            sB[i] = make_longlong2(t[2 * stride + (int64_t)(p0 + k) * wb + j], t[3 * stride + (int64_t)(p0 + k) * wb + j]);
+        }
+        __syncthreads();
+        for (int w = threadIdx.x; w < gp * wa; w += kColThreadsG) {
+            const int kp = w / wa, xc = w - kp * wa, p = p0 + kp;
+            const longlong2* B = sB + kp * wb;
+            const long long ax = t[0 * stride + (int64_t)p * wa + xc];
+            const long long abx = t[1 * stride + (int64_t)p * wa + xc];
+            float acc = 0.0f, cmp = 0.0f;
+            for (int jc = 0; jc < wb; ++jc) {
+                const longlong2 b = B[jc];
+                const long long ua = ax + b.x, ub = abx + b.y;
+                const float fa = (float)((uint32_t)ua >> 8) * 0x1p-24f, ga = 1.0f - fa;
+                const float fb = (float)((uint32_t)ub >> 8) * 0x1p-24f, gb = 1.0f - fb;
+                float s[2][2];
+#pragma unroll
+                for (int db = 0; db < 2; ++db)
+#pragma unroll
+                    for (int da = 0; da < 2; ++da) {
+                        const int xa = (int)(ua >> 32) - kPad + da, xb = (int)(ub >> 32) - kPad + db;
+                        s[db][da] = (xa >= 0 && xa < wa && xb >= 0 && xb < wb) ? __ldg(gbase + (int64_t)xb * ma + xa) : 0.0f;
+                    }
+                const float top = __fmaf_rn(fa, s[0][1], ga * s[0][0]);
+                const float bot = __fmaf_rn(fa, s[1][1], ga * s[1][0]);
+                r4_kahan(acc, cmp, __fmaf_rn(fb, bot, gb * top));
+            }
+            const int64_t o = (((int64_t)p * ha + ya) * hb + yb) * wa + xc;
+            c_hi[o] = acc;
+            c_lo[o] = -cmp;
         }
     }
 }
@@ -265,39 +354,62 @@ Refocus4dLayout refocus4d_layout(int ha, int wa, int hb, int wb, int n_planes) {
 }
 
 namespace {
-// planes per pass of the column stage
-int r4_col_group(int wa, int wb, int np) {
-    int G = wa < kColThreads ? kColThreads / wa : 1;
-    if (G > np) G = np;
-    while (G > 1 && (size_t)G * 2 * wb * sizeof(long long) > 16 * 1024) --G;
-    return G < 1 ? 1 : G;
-}
-size_t r4_box_bytes(int wa, int wb) { return sizeof(float) * (size_t)(wb + 2 * kPad) * (wa + 2 * kPad); }
-constexpr size_t kR4SmemCap = 200 * 1024;
+constexpr size_t kR4SmemCap = 224 * 1024;
+constexpr size_t kR4TableCap = 16 * 1024;
 
-template <bool kSmem, int K>
-cudaError_t launch_cols(const float* g, int np, int G, int ha, int wa, int hb, int wb, const long long* t,
-                        int64_t stride, float* c_hi, float* c_lo, size_t smem, cudaStream_t st) {
+// planes per pass of the column stage, evenly over the passes
+int r4_col_group(int threads, int wa, int wb, int np) {
+    int G = threads / wa;
+    while (G > 1 && (size_t)G * wb * sizeof(longlong2) > kR4TableCap) --G;
+    if (G < 1) G = 1;
+    if (G > np) G = np;
+    const int passes = (np + G - 1) / G;
+    return (np + passes - 1) / passes;
+}
+
+struct ColPlan {
+    int K, WP, threads, G;
+    size_t smem;
+};
+// Rows per CTA (4, 2, 1): as many as fit, while the grid keeps ~4 CTAs per SM of a
+// 152-SM GPU.  K = 0: not even one row's box fits.
+// skew: the sign of alpha - 1 against gamma over the planes (see r4_cols_kernel).
+ColPlan r4_col_plan(int ha, int wa, int hb, int wb, int np, double skew) {
+    for (int K : {4, 2, 1}) {
+        if (K > 1 && (int64_t)hb * ((ha + K - 1) / K) < 4 * 152) continue;
+        const int bank = 32 / K, tight = wa + 2 * kPad;
+        const int want = skew >= 0.0 ? bank - 1 : 1;
+        for (int WP : {tight + (want - tight % bank + bank) % bank, tight}) {
+            const size_t box = (size_t)(wb + 2 * kPad) * WP * K * sizeof(float);
+            for (int threads : {512, 1024}) {
+                const int G = r4_col_group(threads, wa, wb, np);
+                const size_t smem = (size_t)G * wb * sizeof(longlong2) + box;
+                if (smem <= (threads == 512 ? kR4SmemCap / 2 : kR4SmemCap)) return {K, WP, threads, G, smem};
+            }
+        }
+    }
+    return {};
+}
+
+template <int K>
+cudaError_t launch_cols(const ColPlan& c, const float* g, int np, int ha, int wa, int hb, int wb, const long long* t,
+                        int64_t stride, float* c_hi, float* c_lo, cudaStream_t st) {
     static bool attr[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!attr[dev]) {
-        if ((e = cudaFuncSetAttribute(r4_cols_kernel<kSmem, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)kR4SmemCap)) != cudaSuccess)
+        if ((e = cudaFuncSetAttribute(r4_cols_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kR4SmemCap)) !=
+            cudaSuccess)
             return e;
         attr[dev] = true;
     }
     const dim3 grid((unsigned)hb, (unsigned)((ha + K - 1) / K));
-    r4_cols_kernel<kSmem, K><<<grid, kColThreads, smem, st>>>(g, np, G, ha, wa, hb, wb, t, stride, c_hi, c_lo);
+    r4_cols_kernel<K><<<grid, c.threads, c.smem, st>>>(g, np, c.G, ha, wa, hb, wb, c.WP, t, stride, c_hi, c_lo);
     return cudaGetLastError();
 }
 }  // namespace
-
-bool refocus4d_box_fits(int wa, int wb) {
-    return sizeof(long long) * 2 * (size_t)wb + r4_box_bytes(wa, wb) <= kR4SmemCap;
-}
 
 cudaError_t launch_refocus4d_chunk(const float* gamma_f32, int ha, int wa, int hb, int wb, const Plane4Block& coef,
                                    int np, uint8_t* ws, const Refocus4dLayout& L, float* out, cudaStream_t st) {
@@ -307,26 +419,27 @@ cudaError_t launch_refocus4d_chunk(const float* gamma_f32, int ha, int wa, int h
     r4_tables_kernel<<<np, 128, 0, st>>>(coef, np, ha, wa, hb, wb, t, L.stride);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    int G = r4_col_group(wa, wb, np);
-    if (refocus4d_box_fits(wa, wb)) {
-        const size_t box = r4_box_bytes(wa, wb);
-        while (G > 1 && sizeof(long long) * 2 * (size_t)G * wb + box > kR4SmemCap) --G;
-        const size_t tab = sizeof(long long) * 2 * (size_t)G * wb;
-        // boxes per CTA: as many row pairs (4, 2, 1) as fit, while the grid
-        // keeps at least ~4 CTAs per SM of a 152-SM GPU
-        int K = 1;
-        for (int k : {4, 2})
-            if (tab + k * box <= kR4SmemCap && (int64_t)hb * ((ha + k - 1) / k) >= 4 * 152) {
-                K = k;
-                break;
-            }
-        const size_t smem = tab + K * box;
-        if (K == 4) e = launch_cols<true, 4>(gamma_f32, np, G, ha, wa, hb, wb, t, L.stride, c_hi, c_lo, smem, st);
-        else if (K == 2) e = launch_cols<true, 2>(gamma_f32, np, G, ha, wa, hb, wb, t, L.stride, c_hi, c_lo, smem, st);
-        else e = launch_cols<true, 1>(gamma_f32, np, G, ha, wa, hb, wb, t, L.stride, c_hi, c_lo, smem, st);
-    } else {
-        e = launch_cols<false, 1>(gamma_f32, np, G, ha, wa, hb, wb, t, L.stride, c_hi, c_lo,
-                                  sizeof(long long) * 2 * (size_t)G * wb, st);
+    double skew = 0.0;
+    for (int p = 0; p < np; ++p) skew += (coef.c[p][0] - 1.0) * coef.c[p][2];
+    const ColPlan c = r4_col_plan(ha, wa, hb, wb, np, skew);
+    if (c.K == 4) e = launch_cols<4>(c, gamma_f32, np, ha, wa, hb, wb, t, L.stride, c_hi, c_lo, st);
+    else if (c.K == 2) e = launch_cols<2>(c, gamma_f32, np, ha, wa, hb, wb, t, L.stride, c_hi, c_lo, st);
+    else if (c.K == 1) e = launch_cols<1>(c, gamma_f32, np, ha, wa, hb, wb, t, L.stride, c_hi, c_lo, st);
+    else {
+        const int G = r4_col_group(kColThreadsG, wa, wb, np);
+        static bool attr[64] = {};
+        int dev = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+        if (!attr[dev]) {   // angular rows of more than 3072 pixels: a table above 48 KiB
+            if ((e = cudaFuncSetAttribute(r4_cols_global_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)) !=
+                cudaSuccess)
+                return e;
+            attr[dev] = true;
+        }
+        r4_cols_global_kernel<<<dim3((unsigned)hb, (unsigned)ha), kColThreadsG, sizeof(longlong2) * (size_t)G * wb, st>>>(
+            gamma_f32, np, G, ha, wa, hb, wb, t, L.stride, c_hi, c_lo);
+        e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
     const int Gr = wa < kR4Threads ? kR4Threads / wa : 1;
