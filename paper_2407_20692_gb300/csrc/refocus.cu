@@ -30,6 +30,7 @@
 //
 // This file is compiled without FMA contraction: the Kahan steps depend on the
 // written rounding order; the products use explicit fmaf.
+#include <cmath>
 #include <cstring>
 
 #include "kernels.cuh"
@@ -319,6 +320,262 @@ __global__ void __launch_bounds__(kBandThreads, 1) refocus_band_kernel(const __g
     }
 }
 
+// ------------------------------------------------------------ x stage on interleaved rows
+// The same sums (bit for bit) from a copy of Gamma whose rows come four to a group,
+// [slice][group][column, 2 zero columns on either side][4 rows], made once per call:
+// a tap of four rows is one 16-byte shared-memory load that arrives as two packed
+// row pairs, and a unit's band of a slice is one contiguous bulk copy.  Bound by the
+// latency of the shared-memory reads (an ncu capture of the form without the reads
+// ahead: 5 of 9 stall cycles per instruction, read wavefronts at 38% of their rate),
+// so each item's loads are issued one item ahead of its arithmetic (4.58 -> 4.22 ms
+// at 128x128 vs 64x64, 128 planes); 24 warps of 2 planes instead of 16 of 4 were
+// slower (4.78 ms).  Whole call, row-major -> this, one GB300: 128x128 vs 64x64, 128
+// planes 4.35 -> 4.22 ms; 96x96 vs 40x40, 128: 1.36 -> 1.05; 83x83 vs 37x37, 128: 1.16 ->
+// 0.80; 70x50 vs 30x30, 128: 0.53 -> 0.32; 40x40 vs 20x20, 256: 0.31 -> 0.19.
+//
+// Thread t owns column t % wa and the KR rows of row set t / wa (R sets; the CTA has
+// just the warps that R x wa threads need, so odd widths waste no lanes); PT planes
+// per thread, one after the other, so the taps live in registers only while their
+// rows are summed.  Units, staging and release as above.
+struct RowGeom {
+    int32_t ha, wa, hb, wb;
+    int32_t n_planes;
+    int32_t R, n_bands, n_pb;
+    int32_t groups, XP;        // row groups of a slice, columns of a staged group (wa + 4)
+    int32_t band_groups;       // row groups of a full band (R KR / 4)
+    int32_t stages;
+    uint32_t stage_bytes;      // of a full band, a multiple of 128
+    const long long* xcol;     // as BandGeom, staging pad 2
+    const long long* xang;
+    unsigned int* status;
+    unsigned long long timeout_ns;
+};
+
+// [slice][group][wa + 4][4] from [slice][ha][wa], zero columns and rows beyond the slice.
+__global__ void __launch_bounds__(256) refocus_interleave_kernel(const float* __restrict__ src, float4* __restrict__ dst,
+                                                                 int64_t n, int ha, int wa, int groups) {
+    const int XP = wa + 4;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t sg = i / XP;
+        const int x = (int)(i - sg * XP) - 2;
+        const int64_t slice = sg / groups;
+        const int y = (int)(sg - slice * groups) * 4;
+        const float* s = src + (slice * ha + y) * wa + x;
+        float v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[r] = (x >= 0 && x < wa && y + r < ha) ? __ldg(s + (int64_t)r * wa) : 0.0f;
+        dst[i] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+}
+
+__device__ __forceinline__ long long lds64(uint32_t a) {
+    long long v;
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+// 16 bytes of shared memory at a 32-bit shared address + OFF.  Volatile: ordered after
+// the waits that make the data visible and before the release.
+template <int OFF>
+__device__ __forceinline__ ulonglong2 lds128(uint32_t a) {
+    ulonglong2 v;
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2 + %3];" : "=l"(v.x), "=l"(v.y) : "r"(a), "n"(OFF) : "memory");
+    return v;
+}
+
+template <int KR, int PT>
+__global__ void __launch_bounds__(kBandThreads, 1) refocus_rows_kernel(const float* __restrict__ gi, const RowGeom g,
+                                                                       float* __restrict__ ubuf) {
+    constexpr int G4 = KR / 4;                                  // row groups per thread
+    extern __shared__ __align__(128) float sm_raw[];
+    uint8_t* const buf0 = reinterpret_cast<uint8_t*>(sm_raw) +
+                          ((128u - (static_cast<uint32_t>(__cvta_generic_to_shared(sm_raw)) & 127u)) & 127u);
+    __shared__ __align__(8) uint64_t full[kBandMaxStages];
+    __shared__ unsigned int relcnt[kBandMaxStages];
+    // coordinate step per angular column (kept out of registers; whole plane blocks, the surplus 0)
+    __shared__ long long step[kRefocusMaxPlanesPerLaunch + PT];
+
+    const int ha = g.ha, wa = g.wa, hb = g.hb, wb = g.wb, XP = g.XP, stages = g.stages;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const unsigned int n_warps = blockDim.x >> 5;
+    const int rp = tid / wa, c = tid - rp * wa;
+    const bool active = rp < g.R;
+    const int per_br = g.n_pb * g.n_bands;
+    const int n_units = hb * per_br;
+    const int n_mine = (int)blockIdx.x < n_units ? (n_units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const uint32_t total_sl = (uint32_t)n_mine * (uint32_t)wb;
+    const int64_t slice_bytes = (int64_t)g.groups * XP * 16;
+
+    // angular column bc of this CTA's unit k (bc may run on into the units that follow) -> stage s
+    auto issue = [&](int k, int bc, int s) {
+        while (bc >= wb) {
+            bc -= wb;
+            ++k;
+        }
+        const int u = (int)blockIdx.x + k * (int)gridDim.x;
+        const int br = u / per_br, band = (u - br * per_br) % g.n_bands;
+        const int g0 = band * g.band_groups;
+        const uint32_t bytes = (uint32_t)(min(g.band_groups, g.groups - g0) * XP) * 16u;
+        mbar_arrive_expect_tx(&full[s], bytes);
+        bulk_load(buf0 + (size_t)s * g.stage_bytes,
+                  reinterpret_cast<const uint8_t*>(gi) + (int64_t)(br * wb + bc) * slice_bytes + (int64_t)g0 * XP * 16, bytes,
+                  &full[s]);
+    };
+
+    if (tid == 0) {
+        for (int i = 0; i < stages; ++i) {
+            mbar_init(&full[i], 1);
+            relcnt[i] = 0;
+        }
+        fence_barrier_init();
+    }
+    for (int p = tid; p < g.n_planes + PT; p += blockDim.x) step[p] = p < g.n_planes ? __ldg(g.xang + 2 * p + 1) : 0ll;
+    __syncthreads();
+    if (tid == 0)
+        for (int q = 0; q < stages && (uint32_t)q < total_sl; ++q) issue(0, q, q);
+
+    const int hi_b = 2 + wa;      // clamp of a tap's staged column: 0 .. wa + 2
+    uint32_t gs = 0;      // slices of this CTA consumed so far
+    int cs = 0;           // stage of slice gs
+    uint32_t cp = 0;      // phase parity of slice gs in its stage
+    const f32x2 one2 = pk2(1.0f, 1.0f);
+    const uint32_t XP16 = (uint32_t)XP * 16u;
+    const uint32_t ring = smem_u32(buf0) + (uint32_t)(rp * G4) * XP16;   // this thread's rows in stage 0
+    for (int k = 0; k < n_mine; ++k) {
+        const int u = (int)blockIdx.x + k * (int)gridDim.x;
+        const int br = u / per_br, rest = u - br * per_br;
+        const int pblk = rest / g.n_bands, band = rest - pblk * g.n_bands;
+        const int p0 = pblk * PT;
+        const int np = min(PT, g.n_planes - p0);
+        long long X[PT];
+#pragma unroll
+        for (int j = 0; j < PT; ++j) {
+            const int pj = p0 + min(j, np - 1);
+            X[j] = __ldg(g.xcol + (size_t)pj * kBandThreads + c) + __ldg(g.xang + 2 * pj);
+        }
+        // sums of row pairs (2h, 2h + 1) in the two lanes of a packed register
+        f32x2 U[PT][KR / 2], C[PT][KR / 2];
+#pragma unroll
+        for (int j = 0; j < PT; ++j)
+#pragma unroll
+            for (int h = 0; h < KR / 2; ++h) U[j][h] = C[j][h] = 0ull;
+        const uint32_t dsteps = smem_u32(step + p0);
+        for (int bc0 = 0; bc0 < wb; bc0 += 2) {
+            const int nsl = min(2, wb - bc0);
+            const int s0 = cs, s1 = cs + 1 == stages ? 0 : cs + 1;
+            const uint32_t p1 = s1 == 0 ? cp ^ 1u : cp;
+            bool ok = mbar_wait_bounded(&full[s0], cp, nullptr, g.status, g.timeout_ns);
+            if (nsl == 2) ok = ok && mbar_wait_bounded(&full[s1], p1, nullptr, g.status, g.timeout_ns);
+            if (!ok) {   // every thread stops at this same slice
+                if (tid == 0)
+                    for (uint32_t q = gs; q < gs + (uint32_t)stages && q < total_sl; ++q)
+                        mbar_wait_bounded(&full[q % (uint32_t)stages], (q / (uint32_t)stages) & 1u, nullptr, nullptr,
+                                          g.timeout_ns);
+                return;
+            }
+            if (active) {
+                const uint32_t S0 = ring + (uint32_t)s0 * g.stage_bytes, S1 = ring + (uint32_t)s1 * g.stage_bytes;
+                if (nsl == 2) {
+                    // Items (plane, row group, slice) in order; an item's two 16-byte
+                    // loads are issued one item ahead of its arithmetic.
+                    uint32_t pa = 0, pb = 0;
+                    float fa = 0.0f, fb = 0.0f;
+                    long long dn = lds64(dsteps);                // the next plane's step
+                    auto taps = [&](int j) {
+                        const long long ua = X[j];
+                        const long long ub = ua + dn;
+                        X[j] = ub + dn;
+                        pa = S0 + 16u * (uint32_t)__vimin_s32_relu((int)(ua >> 32), hi_b);
+                        pb = S1 + 16u * (uint32_t)__vimin_s32_relu((int)(ub >> 32), hi_b);
+                        fa = (float)((uint32_t)ua >> 8) * 0x1p-24f;
+                        fb = (float)((uint32_t)ub >> 8) * 0x1p-24f;
+                        if (j + 1 < PT) dn = lds64(dsteps + 8u * (uint32_t)(j + 1));
+                    };
+                    taps(0);
+                    ulonglong2 v0 = lds128<0>(pa), v1 = lds128<16>(pa);
+#pragma unroll
+                    for (int j = 0; j < PT; ++j) {
+                        const f32x2 a1 = pk2(fa, fa), a0 = sub2(one2, a1), b1 = pk2(fb, fb), b0 = sub2(one2, b1);
+#pragma unroll
+                        for (int q = 0; q < G4; ++q) {
+                            const ulonglong2 w0 = lds128<0>(pb), w1 = lds128<16>(pb);
+                            const f32x2 tx = fma2(a1, v1.x, mul2(a0, v0.x)), ty = fma2(a1, v1.y, mul2(a0, v0.y));
+                            if (q + 1 < G4) {
+                                pa += XP16;
+                                pb += XP16;
+                            } else if (j + 1 < PT) {
+                                taps(j + 1);
+                            }
+                            if (q + 1 < G4 || j + 1 < PT) {
+                                v0 = lds128<0>(pa);
+                                v1 = lds128<16>(pa);
+                            }
+                            kahan_add2(U[j][2 * q], C[j][2 * q], fma2(b1, w1.x, fma2(b0, w0.x, tx)));
+                            kahan_add2(U[j][2 * q + 1], C[j][2 * q + 1], fma2(b1, w1.y, fma2(b0, w0.y, ty)));
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < PT; ++j) {
+                        const long long ua = X[j];
+                        uint32_t pa = S0 + 16u * (uint32_t)__vimin_s32_relu((int)(ua >> 32), hi_b);
+                        const float fa = (float)((uint32_t)ua >> 8) * 0x1p-24f;
+                        const f32x2 a1 = pk2(fa, fa), a0 = sub2(one2, a1);
+#pragma unroll
+                        for (int q = 0; q < G4; ++q, pa += XP16) {
+                            const ulonglong2 va0 = lds128<0>(pa), va1 = lds128<16>(pa);
+                            kahan_add2(U[j][2 * q], C[j][2 * q], fma2(a1, va1.x, mul2(a0, va0.x)));
+                            kahan_add2(U[j][2 * q + 1], C[j][2 * q + 1], fma2(a1, va1.y, mul2(a0, va0.y)));
+                        }
+                    }
+                }
+            }
+            // release the step's buffers; the last warp to do so refills them
+            __syncwarp();
+            if (lane == 0) {
+                for (int i = 0; i < nsl; ++i) {
+                    const uint32_t q = gs + i;
+                    const int s = i == 0 ? s0 : s1;
+                    __threadfence_block();
+                    if (atomicAdd(&relcnt[s], 1u) == n_warps - 1) {
+                        relcnt[s] = 0;
+                        __threadfence_block();
+                        if (q + stages < total_sl) {
+                            fence_proxy_async_smem();
+                            issue(k, bc0 + i + stages, s);
+                        }
+                    }
+                }
+            }
+            gs += nsl;
+            cs = nsl == 2 ? s1 : s0;
+            cp = nsl == 2 ? p1 : cp;
+            if (++cs == stages) {
+                cs = 0;
+                cp ^= 1u;
+            }
+        }
+        if (active) {
+            const int64_t Ma = (int64_t)ha * wa;
+            const int row0 = band * g.band_groups * 4 + rp * KR;
+#pragma unroll
+            for (int j = 0; j < PT; ++j) {
+                if (j >= np) continue;
+                float* o = ubuf + ((int64_t)(p0 + j) * hb + br) * Ma + c;
+#pragma unroll
+                for (int h = 0; h < KR / 2; ++h) {
+                    float v[2];
+                    unpk2(sub2(U[j][h], C[j][h]), v[0], v[1]);
+#pragma unroll
+                    for (int l = 0; l < 2; ++l) {
+                        const int row = row0 + 2 * h + l;
+                        if (row < ha) o[(int64_t)row * wa] = v[l];
+                    }
+                }
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------ y stage
 // out[p][r][c] = sum over br of wy0 U[p][br][yo][c] + wy1 U[p][br][yo + 1][c],
 // Kahan-added over br in order.  CTA = (RB output rows, plane); the y taps of its
@@ -508,6 +765,69 @@ cudaError_t launch_band(const BandPlan& b, const CUtensorMap* tm, const BandGeom
     }
 }
 
+// The interleaved form: its row sets, rows and planes per thread, and how the call's
+// planes are split into launches.  The copy of Gamma shares the workspace with the
+// x-stage images, so it needs a call of enough planes: the images of a launch's
+// planes and the copy together take the workspace of the row-major form.
+struct RowPlan {
+    bool ok;
+    int KR, PT, R, n_bands, threads, per_sm, band_groups, groups, stages;
+    int chunk;              // planes per launch
+    size_t stage_bytes, smem, copy_off;
+};
+
+RowPlan row_plan(int ha, int wa, int hb, int wb, int n_planes, size_t image_bytes, int sm_count) {
+    RowPlan b{};
+    const size_t Ma = (size_t)ha * wa;
+    b.groups = (ha + 3) / 4;
+    const size_t copy = (size_t)hb * wb * b.groups * (wa + 4) * 16;
+    if (copy + 256 > image_bytes) return b;
+    int64_t most = (int64_t)((image_bytes - copy - 256) / ((size_t)hb * Ma * sizeof(float)));
+    if (most > kRefocusMaxPlanesPerLaunch) most = kRefocusMaxPlanesPerLaunch;
+    const int64_t fewest = n_planes < 16 ? n_planes : 16;
+    if (most < fewest) return b;
+    int launches = (int)((n_planes + most - 1) / most);
+    b.chunk = (n_planes + launches - 1) / launches;
+    if (b.chunk % 4 != 0 && (b.chunk + 3) / 4 * 4 <= most) b.chunk = (b.chunk + 3) / 4 * 4;
+    b.copy_off = ((size_t)b.chunk * hb * Ma * sizeof(float) + 255) / 256 * 256;
+    // 512 threads share an SM (128 registers each), as several CTAs where a CTA is
+    // smaller: row sets with the fewest issue slots for the whole image.  Per two
+    // slices a warp spends about 60 on the stage's waits and release, and a thread per
+    // plane 24 on the taps and 5 per row; fewer resident warps hide less latency.
+    b.KR = 8;
+    b.PT = 4;
+    const int most_t = wa <= 256 ? 256 : kBandThreads, regs_t = kBandThreads;
+    double best = 0.0;
+    for (int R = 1; R * wa <= most_t; ++R) {
+        const int warps = (R * wa + 31) / 32, bands = (ha + R * b.KR - 1) / (R * b.KR);
+        const int per_sm = regs_t / (32 * warps) < 8 ? regs_t / (32 * warps) : 8;
+        const size_t stage = ((size_t)R * b.KR * (wa + 4) * 4 + 127) / 128 * 128;
+        const size_t st = (208 * 1024 / per_sm - 2048) / stage;
+        if (st < 4) continue;
+        const double slots = warps * (60.0 / b.PT + (24 + 5 * b.KR));
+        const double cost = bands * slots * std::sqrt(16.0 / (per_sm * warps));
+        if (b.ok && cost >= best) continue;
+        best = cost;
+        b.ok = true;
+        b.R = R;
+        b.n_bands = bands;
+        b.threads = 32 * warps;
+        b.per_sm = per_sm;
+        b.band_groups = R * b.KR / 4;
+        b.stage_bytes = stage;
+        b.stages = st > kBandMaxStages ? kBandMaxStages : (int)st;
+        b.smem = 128 + (size_t)b.stages * stage;
+    }
+    // Small calls: the row-major form spreads them over more threads (2 rows each for
+    // narrow images) and needs no copy; where a launch has less than two full sets of
+    // warps it is the faster one (21x21 vs 13x13 with 39 planes: 67 us a step against
+    // 94; 22x92 vs 38x38 with 61 planes, which the copy splits into 4 launches: 286
+    // against 312).
+    const int64_t units = (int64_t)hb * ((b.chunk + b.PT - 1) / b.PT) * b.n_bands;
+    if (units * (b.threads / 32) < 2 * (int64_t)sm_count * 16) b.ok = false;
+    return b;
+}
+
 // Output rows per y-stage CTA: its y taps (rows x hb entries) fit in 200 KiB.
 int y_rows_per_cta(int hb) {
     int rb = (int)((200 * 1024) / ((size_t)hb * sizeof(YTap)));
@@ -541,36 +861,48 @@ size_t refocus_ws_bytes(int ha, int wa, int hb, int wb, int n_planes) {
     return bytes + xtables_bytes();
 }
 
-int refocus_launches(int ha, int wa, int n_planes) {
-    const int chunks = (n_planes + kRefocusMaxPlanesPerLaunch - 1) / kRefocusMaxPlanesPerLaunch;
-    return 3 * chunks + (band_plan(ha, wa).pitch ? 1 : 0);
-}
-
 cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, const double* alpha,
                         const double* beta, int n_planes, float* out, void* workspace, int sm_count,
                         unsigned int* status, unsigned long long timeout_ns, cudaStream_t st) {
     const int64_t Ma = (int64_t)ha * wa, Mb = (int64_t)hb * wb;
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    PlaneBlock pb;
     const BandPlan b = band_plan(ha, wa);
-    {
-        if (!b.ok) return cudaErrorInvalidValue;
-        const int per_launch = n_planes < kRefocusMaxPlanesPerLaunch ? n_planes : kRefocusMaxPlanesPerLaunch;
-        float* ubuf = reinterpret_cast<float*>(ws);
+    if (!b.ok) return cudaErrorInvalidValue;
+    const int per_launch = n_planes < kRefocusMaxPlanesPerLaunch ? n_planes : kRefocusMaxPlanesPerLaunch;
+    float* ubuf = reinterpret_cast<float*>(ws);
+    // the workspace: x-stage images and a copy of Gamma, then the x-coordinate tables
+    const size_t copy_off = round256((size_t)per_launch * hb * Ma * sizeof(float));
+    size_t tab_off = copy_off;
+    if (b.pitch) tab_off += round256(Mb * ha * (size_t)b.pitch * sizeof(float));
+    long long* xcol = reinterpret_cast<long long*>(ws + tab_off);
+    long long* xang = reinterpret_cast<long long*>(
+        ws + tab_off + round256((size_t)kRefocusMaxPlanesPerLaunch * kBandThreads * sizeof(long long)));
+    const RowPlan rw = row_plan(ha, wa, hb, wb, n_planes, tab_off, sm_count);
+    cudaError_t e = cudaSuccess;
+    CUtensorMap tm;
+    const float* gi = nullptr;
+    if (rw.ok) {
+        float* copy = reinterpret_cast<float*>(ws + rw.copy_off);
+        const int64_t n = Mb * rw.groups * (wa + 4);
+        int64_t blocks = (n + 255) / 256;
+        if (blocks > 16 * (int64_t)sm_count) blocks = 16 * (int64_t)sm_count;
+        refocus_interleave_kernel<<<(unsigned)blocks, 256, 0, st>>>(gamma_f32, reinterpret_cast<float4*>(copy), n, ha, wa,
+                                                                    rw.groups);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        gi = copy;
+    } else {
         const float* src = gamma_f32;
         int pitch = wa;
         if (b.pitch) {
-            float* copy = reinterpret_cast<float*>(ws + round256((size_t)per_launch * hb * Ma * sizeof(float)));
+            float* copy = reinterpret_cast<float*>(ws + copy_off);
             const int64_t rows = Mb * ha;
             int64_t blocks = (rows * b.pitch + 255) / 256;
             if (blocks > 8 * (int64_t)sm_count) blocks = 8 * (int64_t)sm_count;
             refocus_repack_kernel<<<(unsigned)blocks, 256, 0, st>>>(gamma_f32, copy, rows, wa, b.pitch);
-            cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
             src = copy;
             pitch = b.pitch;
         }
-        CUtensorMap tm;
         if (!b.mode3d) {
             const uint64_t dims[2] = {(uint64_t)wa, (uint64_t)(Mb * ha)};
             const uint64_t strides[1] = {(uint64_t)pitch * sizeof(float)};
@@ -582,19 +914,46 @@ cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, 
             const uint32_t box[3] = {16, (uint32_t)(b.WS / 16), (uint32_t)b.BH};
             if (!make_f32_map(&tm, src, 3, dims, strides, box)) return cudaErrorInvalidValue;
         }
-        const int RB = y_rows_per_cta(hb);
-        size_t tab_off = round256((size_t)per_launch * hb * Ma * sizeof(float));
-        if (b.pitch) tab_off += round256(Mb * ha * (size_t)b.pitch * sizeof(float));
-        long long* xcol = reinterpret_cast<long long*>(ws + tab_off);
-        long long* xang = reinterpret_cast<long long*>(
-            ws + tab_off + round256((size_t)kRefocusMaxPlanesPerLaunch * kBandThreads * sizeof(long long)));
-        for (int p0 = 0; p0 < n_planes; p0 += kRefocusMaxPlanesPerLaunch) {
-            const int np = n_planes - p0 < kRefocusMaxPlanesPerLaunch ? n_planes - p0 : kRefocusMaxPlanesPerLaunch;
-            std::memset(&pb, 0, sizeof(pb));
-            for (int i = 0; i < np; ++i) {
-                pb.alpha[i] = alpha[p0 + i];
-                pb.beta[i] = beta[p0 + i];
-            }
+    }
+    const int RB = y_rows_per_cta(hb);
+    const int chunk = rw.ok ? rw.chunk : kRefocusMaxPlanesPerLaunch;
+    PlaneBlock pb;
+    for (int p0 = 0; p0 < n_planes; p0 += chunk) {
+        const int np = n_planes - p0 < chunk ? n_planes - p0 : chunk;
+        std::memset(&pb, 0, sizeof(pb));
+        for (int i = 0; i < np; ++i) {
+            pb.alpha[i] = alpha[p0 + i];
+            pb.beta[i] = beta[p0 + i];
+        }
+        refocus_xtables_kernel<<<(unsigned)((np * kBandThreads + 255) / 256), 256, 0, st>>>(
+            pb, np, wa, wb, rw.ok ? 2 : b.pad_l, xcol, xang);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (rw.ok) {
+            RowGeom g{};
+            g.ha = ha;
+            g.wa = wa;
+            g.hb = hb;
+            g.wb = wb;
+            g.n_planes = np;
+            g.R = rw.R;
+            g.n_bands = rw.n_bands;
+            g.n_pb = (np + rw.PT - 1) / rw.PT;
+            g.groups = rw.groups;
+            g.XP = wa + 4;
+            g.band_groups = rw.band_groups;
+            g.stages = rw.stages;
+            g.stage_bytes = (uint32_t)rw.stage_bytes;
+            g.xcol = xcol;
+            g.xang = xang;
+            g.status = status;
+            g.timeout_ns = timeout_ns;
+            const int64_t units = (int64_t)hb * g.n_pb * g.n_bands;
+            const int64_t ctas = (int64_t)sm_count * rw.per_sm;
+            const int grid = (int)(units < ctas ? units : ctas);
+            if ((e = set_smem_attr(refocus_rows_kernel<8, 4>, 10, kSmemCap)) != cudaSuccess) return e;
+            refocus_rows_kernel<8, 4><<<grid, rw.threads, rw.smem, st>>>(gi, g, ubuf);
+            e = cudaGetLastError();
+        } else {
             BandGeom g{};
             g.ha = ha;
             g.wa = wa;
@@ -614,23 +973,17 @@ cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, 
             g.xang = xang;
             g.status = status;
             g.timeout_ns = timeout_ns;
-            refocus_xtables_kernel<<<(unsigned)((np * kBandThreads + 255) / 256), 256, 0, st>>>(pb, np, wa, wb, b.pad_l,
-                                                                                               xcol, xang);
-            cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
             const int64_t units = (int64_t)hb * g.n_pb * g.n_bands;
             const int grid = units < sm_count ? (int)units : sm_count;
             e = launch_band(b, &tm, g, pb, ubuf, grid, st);
-            if (e != cudaSuccess) return e;
-            YGeom y{ha, wa, hb, RB, p0};
-            const size_t ysmem = (size_t)RB * hb * sizeof(YTap);
-            e = set_smem_attr(refocus_ystage_kernel, 20, kSmemCap);
-            if (e != cudaSuccess) return e;
-            refocus_ystage_kernel<<<dim3((unsigned)((ha + RB - 1) / RB), (unsigned)np), kYThreads, ysmem, st>>>(
-                ubuf, y, pb, out);
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
         }
+        if (e != cudaSuccess) return e;
+        YGeom y{ha, wa, hb, RB, p0};
+        const size_t ysmem = (size_t)RB * hb * sizeof(YTap);
+        if ((e = set_smem_attr(refocus_ystage_kernel, 20, kSmemCap)) != cudaSuccess) return e;
+        refocus_ystage_kernel<<<dim3((unsigned)((ha + RB - 1) / RB), (unsigned)np), kYThreads, ysmem, st>>>(ubuf, y, pb,
+                                                                                                           out);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
