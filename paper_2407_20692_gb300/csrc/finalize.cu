@@ -10,10 +10,8 @@
 //
 // Division: GB300's FP64 pipe runs at a small fraction of its FP32 rate, and an
 // IEEE double division costs a dozen FP64 instructions.  With the divisor
-// D = N^2 the same for every entry, the kernel takes one FP64 multiply by the
-// host-computed reciprocal (within 2 ulp of the quotient) and then fixes the
-// last bit exactly with 128-bit integer arithmetic: q = M * 2^E is the
-// correctly rounded A / D iff (2M - 1) D <= 2 A 2^-E <= (2M + 1) D, ties to even.
+// D = N^2 the same for every entry, the quotient is one 64-bit high product with a
+// reciprocal formed on the host, rounded in integers (gamma_div.cuh).
 // Numerators of 2^53 or more (possible only for very long acquisitions) take
 // the IEEE division.  Sums handed to cpi_correlate_finalize may come from many
 // accumulating calls, so there (wide != 0) the numerator is formed in 128 bits;
