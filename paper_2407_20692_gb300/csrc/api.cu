@@ -170,9 +170,9 @@ struct CorrPlan {
 
 // split == 0: single correlation (more frame chunks when the tiles alone cannot
 // fill the GPU); split >= 1: member of a batch, split x the minimum chunk count.
-// block_n: output tile width (256; batches may choose 128).
-cpi_status make_plan(const cpi_frames* a, const cpi_frames* b, int64_t n, int sm_count,
-                     CorrPlan* pl, int split = 0, int block_n = 256) {
+// block_n: output tile width, 256 or 128.
+cpi_status make_plan_tiles(const cpi_frames* a, const cpi_frames* b, int64_t n, int sm_count, CorrPlan* pl, int split,
+                           int block_n) {
     cpi_status s = check_frames(a);
     if (s != CPI_OK) return s;
     s = check_frames(b);
@@ -223,6 +223,31 @@ cpi_status make_plan(const cpi_frames* a, const cpi_frames* b, int64_t n, int sm
     p.off_sb = round_up(p.off_sa + (size_t)p.Ma * 8, 256);
     p.ws_bytes = round_up(p.off_sb + (size_t)p.Mb * 8, 1024);
     *pl = p;
+    return CPI_OK;
+}
+
+// Length of the raw-moment launch: its waves of units times a unit's time, in cycles
+// of a 128 x 256 tile's K block (512) and of its epilogue.  A tile of half the width
+// takes 0.62 of the time (measured: 128x128 vs 64x64, N = 50000, 27 waves in 4.32 ms
+// against 14 in 3.64 ms; it reads as much of A from shared memory for half the
+// columns), so it pays where it fills the last wave or the last column tile better.
+double moments_cost(const CorrPlan& p, int sm_count) {
+    const double unit = (double)p.kb_per_chunk * 512.0 + 2500.0;
+    return (double)((p.n_units + sm_count - 1) / sm_count) * unit * (p.block_n == 128 ? 0.62 : 1.0);
+}
+
+// The plan of a single correlation: the tile width with the shorter raw-moment
+// launch (83x83 vs 37x37, N = 17321: 324 tiles of 256 columns in 3 waves, 594 of 128
+// in 4; 320 -> 275 us).  Narrow tiles never need more partial slots.
+cpi_status make_plan(const cpi_frames* a, const cpi_frames* b, int64_t n, int sm_count, CorrPlan* pl) {
+    CorrPlan wide, narrow;
+    cpi_status s = make_plan_tiles(a, b, n, sm_count, &wide, 0, 256);
+    if (s != CPI_OK) return s;
+    *pl = wide;
+    s = make_plan_tiles(a, b, n, sm_count, &narrow, 0, 128);
+    if (s == CPI_OK && narrow.ws_bytes <= wide.ws_bytes &&
+        moments_cost(narrow, sm_count) < 0.95 * moments_cost(wide, sm_count))
+        *pl = narrow;
     return CPI_OK;
 }
 
@@ -398,7 +423,7 @@ cpi_status make_batch_plan(const cpi_batch_item* items, int n, int sm, BatchShap
         cpi_status s = check_batch_item(b);
         if (s != CPI_OK) return s;
         BatchItemPlan& ip = bp->it[i];
-        s = make_plan(&b.a, &b.b, b.n_frames, sm, &ip.pl, shape.split, shape.block_n);
+        s = make_plan_tiles(&b.a, &b.b, b.n_frames, sm, &ip.pl, shape.split, shape.block_n);
         if (s != CPI_OK) return s;
         ip.ws_off = off;
         off = round_up(off + ip.pl.ws_bytes, 1024);

@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint64_t tmo = L.timeout_ns;
     unsigned int* const status = L.status;
 
@@ -239,8 +239,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             // ---------------------------------------------------------- MMA issuer
+            // The whole warp runs the loop and one lane issues: the descriptors
+            // stay in uniform registers.
             // The tensor pipe takes one 128 x 256 x 16 (BF16) or x 32 (E2M1) MMA
             // per 128 cycles only while this thread issues the next one within
             // that time, so the loop keeps its per-K-block work to a few adds:
@@ -249,6 +251,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             constexpr uint32_t idesc = idesc_f32acc<kBf16>(kBlockM, C::kBlockN);
             const uint64_t da0 = sdesc_kmajor_sw128(smem_u32(sA));
             const uint64_t db0 = sdesc_kmajor_sw128(smem_u32(sB));
+            const uint32_t on = elect_one() ? 1u : 0u;
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
@@ -263,14 +266,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const bool seg_start = seg_left == 0;
                     if (seg_start) {
                         seg_left = min(kb_per_seg, nkb - i);
-                        if (!mbar_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, status, tmo)) {
+                        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, status, tmo))) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
                     }
                     --seg_left;
-                    if (!mbar_wait_bounded(&full[stage], phase, abort_flag, status, tmo)) {
+                    if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[stage], phase, abort_flag, status, tmo))) {
                         ok = false;
                         break;
                     }
@@ -281,17 +284,17 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                     for (int k = 0; k < kRowBytes / 32; ++k) {
                         // advance the start address by 32 bytes (2 x 16-byte units) per MMA
-                        umma_f32<kBf16>(d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc,
-                                        (seg_start && k == 0) ? 0u : 1u);
+                        umma_f32_warp<kBf16>(on, d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc,
+                                             (seg_start && k == 0) ? 0u : 1u);
                     }
                     issued_any = true;
-                    umma_commit(&empty[stage]);
+                    umma_commit_warp(on, &empty[stage]);
                     if (++stage == C::kStages) {
                         stage = 0;
                         phase ^= 1;
                     }
                     if (seg_left == 0) {   // segment (BF16) or unit (E2M1) done: hand the accumulator over
-                        umma_commit(&tfull[acc]);
+                        umma_commit_warp(on, &tfull[acc]);
                         if (++acc == C::kAcc) {
                             acc = 0;
                             acc_phase ^= 1;
@@ -300,7 +303,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
             if (!ok && issued_any) {
-                umma_commit(drain);
+                umma_commit_warp(on, drain);
                 mbar_wait_bounded(drain, 0, nullptr, nullptr, tmo);
             }
         }
