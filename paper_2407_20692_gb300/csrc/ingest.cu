@@ -4,8 +4,7 @@
 // packed one bit per pixel (Section 2 of the paper) or one byte per pixel.  The
 // raw-moment contraction sums over frames, so each operand row must hold one
 // pixel's values over consecutive frames (K-major):
-//   - 1-bit frames whose region rows are whole 32-pixel words apart ->
-//     FP4 E2M1 values packed two per byte (0x0 / 0x2 = 1.0; frame 2j in the low
+//   - 1-bit frames that start on 4-byte words -> FP4 E2M1 values packed two per byte (0x0 / 0x2 = 1.0; frame 2j in the low
 //     nibble of byte j), ingest_bits_kernel: a block of frames staged word-wise
 //     in shared memory, transposed 32 x 32 bits per warp;
 //   - 8-bit frames with 4-pixel aligned regions -> BF16 (integers 0..255 are
@@ -259,12 +258,12 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t w, int lane) {
     return w;
 }
 
-// Binary frames whose region rows are a multiple of 32 pixels wide, with
-// 4-byte aligned frames.  CTA = (region, chunk of kWC frame words) x block of
+// Binary frames with 4-byte aligned frames.  CTA = (region, chunk of kWC frame words) x block of
 // kFB frames.  Words w0 .. w0 + kWC of every frame of the block are loaded with
 // coalesced 4-byte loads into shared memory, in rows of kWP words (kWP odd: a
 // warp reading one word of 32 frames touches 32 banks).  Each warp then takes
-// whole 32-pixel tiles of the region whose first word lies in the chunk: per 32
+// 32-pixel tiles of the region's rows (the last of a row may hold fewer pixels,
+// whose operand rows alone are written) whose first word lies in the chunk: per 32
 // frames, lane i funnel-shifts its frame's 32 pixel bits out of two words, the
 // warp transposes the 32 x 32 bit block (lane j then holds pixel j over the 32
 // frames), and each bit becomes one E2M1 nibble (0x2 = 1.0; 8 bits -> 8 nibbles
@@ -327,7 +326,7 @@ __global__ void __launch_bounds__(256) ingest_bits_kernel(FramesDev A, FramesDev
     __syncthreads();
 
     // rows with a tile whose first bit e0 = (y0 + y) rs + x0 + 32 xt lies in the chunk
-    const int ntx = d.width >> 5;
+    const int ntx = (d.width + 31) >> 5;
     const int64_t rs = d.row_stride, lo_bit = w0 << 5, hi_bit = (w0 + kWC) << 5;
     int64_t ylo = -floor_div(-(lo_bit - d.x0 - 32 * (int64_t)(ntx - 1)), rs) - d.y0;
     int64_t yhi = floor_div(hi_bit - 1 - d.x0, rs) - d.y0;
@@ -364,14 +363,16 @@ __global__ void __launch_bounds__(256) ingest_bits_kernel(FramesDev A, FramesDev
         }
         __syncwarp();
         const int64_t p0 = y * d.width + 32 * (int64_t)xt;
+        const int n_px = min(32, d.width - 32 * xt);
 #pragma unroll
         for (int k = 0; k < 32 * (kFB / 2) / 16 / 32; ++k) {
             const int idx = k * 32 + lane, r = idx / (kFB / 32), c16 = idx % (kFB / 32);
-            *reinterpret_cast<uint4*>(op + (p0 + r) * kstride_bytes + f0 / 2 + c16 * 16) =
-                *reinterpret_cast<const uint4*>(st + r * kStageRow + c16 * 16);
+            if (r < n_px)
+                *reinterpret_cast<uint4*>(op + (p0 + r) * kstride_bytes + f0 / 2 + c16 * 16) =
+                    *reinterpret_cast<const uint4*>(st + r * kStageRow + c16 * 16);
         }
         __syncwarp();
-        if (cnt) atomicAdd(reinterpret_cast<unsigned long long*>(s + p0 + lane), (unsigned long long)cnt);
+        if (cnt && lane < n_px) atomicAdd(reinterpret_cast<unsigned long long*>(s + p0 + lane), (unsigned long long)cnt);
     }
 }
 
@@ -379,7 +380,7 @@ __global__ void __launch_bounds__(256) ingest_bits_kernel(FramesDev A, FramesDev
 
 // Conditions of the word-load path for binary frames.
 static bool bits_fast_ok(const FramesDev& d) {
-    return d.bits == 1 && d.width % 32 == 0 && d.frame_stride % 4 == 0 &&
+    return d.bits == 1 && d.width >= 8 && d.frame_stride % 4 == 0 &&
            reinterpret_cast<uintptr_t>(d.data) % 4 == 0;
 }
 // Conditions of the 4-pixel path for 8-bit frames.
