@@ -272,7 +272,7 @@ void fill_problem(const CorrPlan& pl, int32_t* part, int unit_begin, MomentsProb
 
 cpi_status run_stage(int stage, const CorrPlan& pl, const cpi_frames* a, const cpi_frames* b,
                      int accumulate, int64_t* s_ab, int64_t* s_a, int64_t* s_b, double* gamma,
-                     float* gamma_f32, void* ws, DeviceInfo* dev, cudaStream_t st, int add_partial = 0) {
+                     float* gamma_f32, void* ws, DeviceInfo* dev, cudaStream_t st, bool chain, int add_partial = 0) {
     uint8_t* w = static_cast<uint8_t*>(ws);
     uint8_t* op_a = w + pl.off_a;
     uint8_t* op_b = w + pl.off_b;
@@ -281,14 +281,8 @@ cpi_status run_stage(int stage, const CorrPlan& pl, const cpi_frames* a, const c
     if (s_a == nullptr) s_a = reinterpret_cast<int64_t*>(w + pl.off_sa);
     if (s_b == nullptr) s_b = reinterpret_cast<int64_t*>(w + pl.off_sb);
     if (stage == CPI_STAGE_INGEST) {
-        if (!accumulate) {
-            cudaError_t e = cudaMemsetAsync(s_a, 0, (size_t)pl.Ma * 8, st);
-            if (e == cudaSuccess) e = cudaMemsetAsync(s_b, 0, (size_t)pl.Mb * 8, st);
-            if (e != cudaSuccess) return CPI_ERR_CUDA;
-        }
-        if (pl.bf16 && cudaMemsetAsync(vmax, 0, 2 * sizeof(uint32_t), st) != cudaSuccess) return CPI_ERR_CUDA;
         return cuda_status(launch_ingest(pl.bf16, to_dev(a), to_dev(b), pl.n, pl.kstride_bytes,
-                                         op_a, op_b, s_a, s_b, pl.bf16 ? vmax : nullptr, st));
+                                         op_a, op_b, s_a, s_b, pl.bf16 ? vmax : nullptr, accumulate == 0, st));
     }
     if (stage == CPI_STAGE_MOMENTS) {
         CUtensorMap tm_a, tm_b;
@@ -305,11 +299,11 @@ cpi_status run_stage(int stage, const CorrPlan& pl, const cpi_frames* a, const c
         L.n_units = pl.n_units;
         L.status = dev->status;
         L.timeout_ns = g_timeout_ns;
-        return cuda_status(launch_moments(pl.bf16, pl.block_n, L, dev->sm_count, st));
+        return cuda_status(launch_moments(pl.bf16, pl.block_n, L, dev->sm_count, chain, st));
     }
     if (stage == CPI_STAGE_FOLD) {
         return cuda_status(launch_fold(part, pl.n_chunks, pl.Ma, pl.Mb, s_ab, accumulate, s_ab != nullptr ? 1 : 0,
-                                       s_a, s_b, pl.n, gamma, gamma_f32, st));
+                                       s_a, s_b, pl.n, gamma, gamma_f32, st, chain));
     }
     return CPI_ERR_INVALID_ARG;
 }
@@ -338,7 +332,7 @@ cpi_status correlate_common(const int32_t* stages, int n_stages, const cpi_frame
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     for (int i = 0; i < n_stages; ++i) {
         s = run_stage(stages[i], pl, a, b, accumulate, s_ab, s_a, s_b, gamma, gamma_f32, ws, dev,
-                      st, add_partial);
+                      st, i > 0, add_partial);
         if (s != CPI_OK) return s;
     }
     return CPI_OK;
@@ -543,7 +537,7 @@ cpi_status run_batch(const cpi_batch_item* items, const BatchPlan& bp, uint8_t* 
         [&](int i, cudaStream_t cs) {
             const cpi_batch_item& b = items[i];
             return run_stage(CPI_STAGE_INGEST, bp.it[i].pl, &b.a, &b.b, 0, b.s_ab, b.s_a, b.s_b, b.gamma,
-                             b.gamma_f32, ws + bp.it[i].ws_off, dev, cs);
+                             b.gamma_f32, ws + bp.it[i].ws_off, dev, cs, false);
         },
         st);
     if (s != CPI_OK) return s;
@@ -558,7 +552,7 @@ cpi_status run_batch(const cpi_batch_item* items, const BatchPlan& bp, uint8_t* 
         [&](int i, cudaStream_t cs) {
             const cpi_batch_item& b = items[i];
             cpi_status r = run_stage(CPI_STAGE_FOLD, bp.it[i].pl, &b.a, &b.b, 0, b.s_ab, b.s_a, b.s_b, b.gamma,
-                                     b.gamma_f32, ws + bp.it[i].ws_off, dev, cs);
+                                     b.gamma_f32, ws + bp.it[i].ws_off, dev, cs, false);
             if (r != CPI_OK || b.n_planes == 0) return r;
             return run_refocus(b.gamma_f32, b.a.height, b.a.width, b.b.height, b.b.width, b.planes, b.n_planes,
                                b.refocus_out, ws + bp.it[i].rws_off, bp.it[i].rws_bytes, cs);
@@ -695,7 +689,7 @@ cpi_status tuned_shape(const cpi_batch_item* items, int n, uint8_t* ws, DeviceIn
         for (int i = 0; i < n && s == CPI_OK; ++i)
             s = run_stage(CPI_STAGE_INGEST, bp.it[i].pl, &items[i].a, &items[i].b, 0, items[i].s_ab,
                           items[i].s_a, items[i].s_b, items[i].gamma, items[i].gamma_f32,
-                          ws + bp.it[i].ws_off, dev, st);
+                          ws + bp.it[i].ws_off, dev, st, false);
         if (s != CPI_OK) break;
         s = launch_batch_moments(items, bp, ws, dev, st);                 // warm-up
         if (s != CPI_OK) break;
@@ -759,7 +753,7 @@ cpi_status acq_flush(Acquisition* q) {
     const int64_t ma = (int64_t)q->a.height * q->a.width, mb = (int64_t)q->b.height * q->b.width;
     const int32_t* part = reinterpret_cast<const int32_t*>(q->ws + q->off_part);
     const cudaError_t e = launch_fold(part, q->n_chunks, ma, mb, q->s_ab, 1, 1, q->s_a, q->s_b, q->n_done, nullptr,
-                                      nullptr, q->compute, 0);
+                                      nullptr, q->compute, false, 0);
     if (e != cudaSuccess) return CPI_ERR_CUDA;
     q->deferred = 0;
     return CPI_OK;
@@ -848,7 +842,7 @@ cpi_status cpi_correlate_finalize(const int64_t* s_ab, const int64_t* s_a, const
     if (n_total > ((int64_t)1 << 31) - 1) return CPI_ERR_OVERFLOW;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     return cuda_status(launch_fold(nullptr, 0, m_a, m_b, const_cast<int64_t*>(s_ab), 1, 0, s_a, s_b,
-                                   n_total, gamma, gamma_f32, st, 1));
+                                   n_total, gamma, gamma_f32, st, false, 1));
 }
 
 size_t cpi_refocus_workspace_size(int32_t ha, int32_t wa, int32_t hb, int32_t wb,

@@ -118,6 +118,8 @@ __device__ __forceinline__ void mask8(float* v, const uint4& m) {
 // by the consumer).
 __global__ void __launch_bounds__(512) dnf_sumsq_kernel(const float* __restrict__ g, int64_t n,
                                                         double* __restrict__ part) {
+    dep_wait();
+    dep_launch();
     __shared__ double red[512];
     double acc = 0.0;
     const int64_t step = (int64_t)gridDim.x * 512;
@@ -151,6 +153,8 @@ __global__ void __launch_bounds__(kStackThreads) dnf_stack_kernel(
     const DnFlat g, const float* __restrict__ gamma, const double* __restrict__ part, int nparts, int64_t n, int hb,
     int wb, const float* __restrict__ model, int stack_blocks, float* __restrict__ scale_out, uint8_t* __restrict__ xin,
     const Margins mg, int w_elems, __nv_bfloat16* __restrict__ wt) {
+    dep_wait();
+    dep_launch();
     if ((int)blockIdx.x >= stack_blocks) {
         const int i = ((int)blockIdx.x - stack_blocks) * kStackThreads + (int)threadIdx.x;
         if (i >= w_elems) return;
@@ -306,6 +310,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) dnf_conv_kernel(const DnFlat 
         tmem_alloc(tmem_slot, kCols);
         tmem_relinquish();
     }
+    dep_wait();
+    dep_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -544,6 +550,8 @@ constexpr int ex_unit(int cout) { return cout == 1 ? 1024 : 512; }
 template <int CIN, int COUT, int MODE>
 __global__ void __launch_bounds__(kExThreads, 2) dnf_conv_exact_kernel(const DnFlat g, const ConvArgs a,
                                                                        const float* __restrict__ w) {
+    dep_wait();
+    dep_launch();
     constexpr int U = ex_unit(COUT), KC = CIN == 9 ? 2 : 4;
     constexpr int WS = COUT == 1 ? 12 : 9 * COUT;               // weights per input channel
     extern __shared__ __align__(16) float sm_ex[];
@@ -709,6 +717,8 @@ __global__ void __launch_bounds__(kTopThreads) dnf_top_grad_kernel(const DnFlat 
                                                                    const float* __restrict__ w3, uint8_t* a3,
                                                                    uint8_t* __restrict__ lo_out,
                                                                    float* __restrict__ bias_part) {
+    dep_wait();
+    dep_launch();
     __shared__ __align__(16) float sw[9][32];
     __shared__ float bred[kTopThreads / 32][32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -848,6 +858,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
         tmem_alloc(tmem_slot, kTmemCols);
         tmem_relinquish();
     }
+    dep_wait();
+    dep_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -981,6 +993,8 @@ __global__ void __launch_bounds__(256) dnf_wgrad_reduce_kernel(const float* __re
                                                                const float* __restrict__ bias_part, int nbias,
                                                                const double* __restrict__ loss_part, int nloss, int64_t n,
                                                                float* __restrict__ grad, float* __restrict__ loss) {
+    dep_wait();
+    dep_launch();
     constexpr int NB = COUT == 32 ? 64 : 16, kCols = 3 * NB, kRows = 3 * KC * 8;
     __shared__ float red[8][32];
     const int co = threadIdx.x & 31, grp = threadIdx.x >> 5;
@@ -1021,6 +1035,10 @@ __global__ void __launch_bounds__(256) dnf_wgrad_reduce_kernel(const float* __re
 }
 
 // ------------------------------------------------------------------ host
+// Short lines gain from kernels placed ahead (42x64 vs 12x9: 86 -> 77 us a call); on
+// long ones the gaps do not count and it costs (64x64 vs 32x32: 514 -> 546 us).
+bool in_chain(const DnFlat& g) { return g.Q < (1u << 20); }
+
 template <typename K>
 cudaError_t allow_smem(K kernel, bool (&done)[64]) {
     int dev = 0;
@@ -1069,8 +1087,8 @@ cudaError_t launch_conv(DnFlat g, ConvArgs a, int sm_count, cudaStream_t st, int
     if (a.stages < 2) return cudaErrorInvalidValue;
     const int grid = g.n_units < sm_count ? g.n_units : sm_count;
     if (ctas) *ctas = grid;
-    dnf_conv_kernel<KC, NOUT, MODE><<<grid, kConvThreads, fixed + a.stages * stage, st>>>(g, a);
-    return cudaGetLastError();
+    return launch_kernel(in_chain(g), dnf_conv_kernel<KC, NOUT, MODE>, grid, kConvThreads, fixed + a.stages * stage, st,
+        g, a);
 }
 
 // The forward layer CIN -> COUT on whichever unit the width takes.
@@ -1088,8 +1106,7 @@ cudaError_t launch_forward(DnFlat g, const ConvArgs& a, const float* w, int sm_c
     int grid = (MODE == kTrain ? 1 : 2) * sm_count;
     if (g.n_units < grid) grid = g.n_units;
     if (ctas) *ctas = grid;
-    dnf_conv_exact_kernel<CIN, COUT, MODE><<<grid, kExThreads, smem, st>>>(g, a, w);
-    return cudaGetLastError();
+    return launch_kernel(in_chain(g), dnf_conv_exact_kernel<CIN, COUT, MODE>, grid, kExThreads, smem, st, g, a, w);
 }
 
 template <int CIN, int KC, int COUT>
@@ -1117,11 +1134,10 @@ cudaError_t launch_wgrad(const DnFlat& g, WgArgs a, const float* bias_part, int 
     a.n_units = (int)(((int64_t)g.Q + U - 1) / U);
     int grid = a.n_units < sm_count ? a.n_units : sm_count;
     if (grid > kDnMaxCtas) grid = kDnMaxCtas;
-    dnf_wgrad_kernel<KC, NB><<<grid, kWgThreads, 256 + a.stages * stage + a.slack, st>>>(g, a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    dnf_wgrad_reduce_kernel<CIN, KC, COUT><<<9 * CIN + 1, 256, 0, st>>>(a.part, grid, bias_part, nbias, loss_part, nloss, n,
-                                                                        grad, loss);
-    return cudaGetLastError();
+    e = launch_kernel(in_chain(g), dnf_wgrad_kernel<KC, NB>, grid, kWgThreads, 256 + a.stages * stage + a.slack, st, g, a);
+    if (e != cudaSuccess) return e;
+    return launch_kernel(in_chain(g), dnf_wgrad_reduce_kernel<CIN, KC, COUT>, 9 * CIN + 1, 256, 0, st, a.part, grid,
+        bias_part, nbias, loss_part, nloss, n, grad, loss);
 }
 
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
@@ -1130,16 +1146,14 @@ cudaError_t launch_inputs(const DnFlat& g, const float* gamma_in, const float* m
                           uint8_t* xin, const Margins& mg, int w_elems, int sm_count, cudaStream_t st) {
     const int64_t n = (int64_t)hb * wb * g.H * g.W;
     double* sums = reinterpret_cast<double*>(ws + g.sums);
-    dnf_sumsq_kernel<<<kDnSumBlocks, 512, 0, st>>>(gamma_in, n, sums);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_kernel(false, dnf_sumsq_kernel, kDnSumBlocks, 512, 0, st, gamma_in, n, sums);
     if (e != cudaSuccess) return e;
     const int64_t want = (g.PL + kStackThreads - 1) / kStackThreads;
     const int sblocks = (int)(want < 16 * (int64_t)sm_count ? want : 16 * (int64_t)sm_count);
     const int wblocks = (w_elems + kStackThreads - 1) / kStackThreads;
-    dnf_stack_kernel<<<sblocks + wblocks, kStackThreads, 0, st>>>(
-        g, gamma_in, sums, kDnSumBlocks, n, hb, wb, model, sblocks, reinterpret_cast<float*>(ws + g.scale), xin, mg, w_elems,
+    return launch_kernel(in_chain(g), dnf_stack_kernel, sblocks + wblocks, kStackThreads, 0, st, g, gamma_in, sums,
+        kDnSumBlocks, n, hb, wb, model, sblocks, reinterpret_cast<float*>(ws + g.scale), xin, mg, w_elems,
         reinterpret_cast<__nv_bfloat16*>(ws + g.wt));
-    return cudaGetLastError();
 }
 
 }  // namespace
@@ -1246,15 +1260,15 @@ cudaError_t dn_flat_grad(const DnFlat& g, const float* model, const float* gamma
     if (e == cudaSuccess) {
         const int64_t blocks = ((int64_t)g.Q + kTopPixels - 1) / kTopPixels;
         nb[2] = (int)(blocks < kTopCtas ? blocks : kTopCtas);
-        dnf_top_grad_kernel<<<nb[2], kTopThreads, 0, st>>>(g, rec, model + kPW3, act[2], lo[0], bpart[2]);
-        e = cudaGetLastError();
+        e = launch_kernel(in_chain(g), dnf_top_grad_kernel, nb[2], kTopThreads, 0, st, g, rec, model + kPW3, act[2],
+            lo[0], bpart[2]);
     }
     const uint8_t* wtb = wt + 2 * kWFwdElems;
     for (int l = 2; l >= 1; --l) {
         w.in = act[l - 1], w.d_hi = act[l], w.d_lo = lo[l & 1];
         if (e == cudaSuccess)
-            e = launch_wgrad<32, 4, 32>(g, w, bpart[l], nb[l], nullptr, 0, n, grad + (l == 2 ? kPW2 : kPW1), nullptr, sm_count,
-                                        st);
+            e = launch_wgrad<32, 4, 32>(g, w, bpart[l], nb[l], nullptr, 0, n, grad + (l == 2 ? kPW2 : kPW1), nullptr,
+                sm_count, st);
         ConvArgs b{};
         b.status = status;
         b.timeout_ns = timeout_ns;

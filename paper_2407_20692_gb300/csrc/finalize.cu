@@ -21,6 +21,7 @@
 // step, through a shared-memory transpose.
 #include "gamma_div.cuh"
 #include "kernels.cuh"
+#include "ptx.cuh"
 
 namespace cpi {
 namespace {
@@ -40,6 +41,8 @@ __global__ void __launch_bounds__(256, 4) fold_kernel(const int32_t* __restrict_
                                                    const int64_t* __restrict__ s_b,
                                                    const GammaDiv gd, int wide, double* gamma,
                                                    float* gamma_f32) {
+    dep_wait();
+    dep_launch();
     __shared__ float tile[kTile][kTile + 1];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;    // 32 x 8
     const Idx b = (Idx)blockIdx.x * kTile + tx;
@@ -96,19 +99,13 @@ __global__ void __launch_bounds__(256, 4) fold_kernel(const int32_t* __restrict_
 cudaError_t launch_fold(const int32_t* partial, int n_chunks, int64_t M, int64_t N,
                         int64_t* s_ab, int accumulate, int write_sab, const int64_t* s_a,
                         const int64_t* s_b, int64_t n_frames, double* gamma, float* gamma_f32,
-                        cudaStream_t st, int wide) {
+                        cudaStream_t st, bool chain, int wide) {
     const int64_t gx = (N + kTile - 1) / kTile, gy = (M + kTile - 1) / kTile;
     const unsigned gyl = (unsigned)(gy < 65535 ? gy : 65535);
     const int64_t span = M * N * (n_chunks > 1 ? n_chunks : 1) + (int64_t)kTile * (M + N);
-    if (span < ((int64_t)1 << 31))
-        fold_kernel<int32_t><<<dim3((unsigned)gx, gyl), 256, 0, st>>>(
-            partial, n_chunks, M, N, s_ab, accumulate, write_sab, s_a, s_b, make_gamma_div(n_frames), wide, gamma,
-            gamma_f32);
-    else
-        fold_kernel<int64_t><<<dim3((unsigned)gx, gyl), 256, 0, st>>>(
-            partial, n_chunks, M, N, s_ab, accumulate, write_sab, s_a, s_b, make_gamma_div(n_frames), wide, gamma,
-            gamma_f32);
-    return cudaGetLastError();
+    return launch_kernel(chain, span < ((int64_t)1 << 31) ? fold_kernel<int32_t> : fold_kernel<int64_t>,
+        dim3((unsigned)gx, gyl), 256, 0, st, partial, n_chunks, M, N, s_ab, accumulate, write_sab, s_a, s_b,
+        make_gamma_div(n_frames), wide, gamma, gamma_f32);
 }
 
 }  // namespace cpi

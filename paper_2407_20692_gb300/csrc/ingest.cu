@@ -21,6 +21,7 @@
 // S_a = sum_i A_i (Eq. (1), second term) with exact int64 atomics.
 
 #include "kernels.cuh"
+#include "ptx.cuh"
 
 namespace cpi {
 namespace {
@@ -31,11 +32,24 @@ __device__ __forceinline__ uint32_t load_pixel(const FramesDev& d, const uint8_t
     return d.bits == 8 ? (uint32_t)v : ((uint32_t)v >> sh) & 1u;
 }
 
+// Marginal sums and maxima to 0 in one launch.
+__global__ void __launch_bounds__(256) ingest_zero_kernel(int64_t* s_a, int64_t na, int64_t* s_b, int64_t nb,
+                                                          uint32_t* vmax) {
+    dep_wait();
+    dep_launch();
+    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
+    if (i < na) s_a[i] = 0;
+    else if (i < na + nb) s_b[i - na] = 0;
+    if (vmax != nullptr && i < 2) vmax[i] = 0;
+}
+
 template <bool kBf16>
 __global__ void __launch_bounds__(256) ingest_kernel(FramesDev A, FramesDev B, int64_t n_frames,
                                                      int64_t kstride_bytes, uint8_t* op_a,
                                                      uint8_t* op_b, int64_t* s_a, int64_t* s_b,
                                                      int tiles_a, uint32_t* vmax) {
+    dep_wait();
+    dep_launch();
     constexpr int kFramesPerWarp = kBf16 ? 16 : 32;   // 32 operand bytes per pixel per warp
     const bool is_a = (int)blockIdx.x < tiles_a;
     const FramesDev d = is_a ? A : B;
@@ -159,6 +173,8 @@ __device__ __forceinline__ uint32_t x4_prmt(uint32_t a, uint32_t b, uint32_t sel
 __global__ void __launch_bounds__(256) ingest_u8x4_kernel(FramesDev A, FramesDev B, int64_t n_frames,
                                                           int64_t kstride_bytes, uint8_t* op_a, uint8_t* op_b,
                                                           int64_t* s_a, int64_t* s_b, int tiles_a, uint32_t* vmax) {
+    dep_wait();
+    dep_launch();
     __shared__ __align__(16) uint8_t tile_s[kX4Pixels * kX4Frames * 2];   // [pixel][16 chunks of 16 B], swizzled
     __shared__ uint32_t part[8][kX4Pixels];
     __shared__ uint32_t wmax[8];
@@ -290,6 +306,8 @@ __host__ __device__ inline int64_t region_last_word(const FramesDev& d) {
 __global__ void __launch_bounds__(256) ingest_bits_kernel(FramesDev A, FramesDev B, int64_t n_frames, int64_t f_base,
                                                           int64_t kstride_bytes, uint8_t* op_a, uint8_t* op_b,
                                                           int64_t* s_a, int64_t* s_b, int chunks_a) {
+    dep_wait();
+    dep_launch();
     extern __shared__ __align__(16) uint8_t smem_bits[];
     uint32_t* S = reinterpret_cast<uint32_t*>(smem_bits);                       // [kFB][kWP]
     const bool is_a = (int)blockIdx.x < chunks_a;
@@ -390,8 +408,16 @@ static bool u8x4_ok(const FramesDev& d) {
 }
 cudaError_t launch_ingest(bool bf16, const FramesDev& a, const FramesDev& b, int64_t n_frames,
                           int64_t kstride_bytes, uint8_t* op_a, uint8_t* op_b, int64_t* s_a,
-                          int64_t* s_b, uint32_t* vmax, cudaStream_t st) {
+                          int64_t* s_b, uint32_t* vmax, bool zero_sums, cudaStream_t st) {
     const int64_t Ma = (int64_t)a.height * a.width, Mb = (int64_t)b.height * b.width;
+    const bool zeroed = zero_sums || vmax != nullptr;
+    if (zeroed) {
+        const int64_t na = zero_sums ? Ma : 0, nb = zero_sums ? Mb : 0;
+        const int64_t n = na + nb > 2 ? na + nb : 2;
+        const cudaError_t e = launch_kernel(false, ingest_zero_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, st,
+            s_a, na, s_b, nb, vmax);
+        if (e != cudaSuccess) return e;
+    }
     const int tiles_a = (int)((Ma + kIngestPixels - 1) / kIngestPixels);
     const int tiles_b = (int)((Mb + kIngestPixels - 1) / kIngestPixels);
     if (!bf16 && bits_fast_ok(a) && bits_fast_ok(b) && (2 * kstride_bytes) % kFB == 0) {
@@ -410,9 +436,9 @@ cudaError_t launch_ingest(bool bf16, const FramesDev& a, const FramesDev& b, int
         const int64_t blocks = 2 * kstride_bytes / kFB;   // two E2M1 frames per byte
         for (int64_t y0 = 0; y0 < blocks; y0 += 65535) {   // grid.y limit
             const int64_t ny = blocks - y0 < 65535 ? blocks - y0 : 65535;
-            ingest_bits_kernel<<<dim3((unsigned)(chunks_a + chunks_b), (unsigned)ny), 256, kBitsSmem, st>>>(
-                a, b, n_frames, y0 * kFB, kstride_bytes, op_a, op_b, s_a, s_b, chunks_a);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if ((e = launch_kernel(zeroed, ingest_bits_kernel, dim3((unsigned)(chunks_a + chunks_b), (unsigned)ny), 256,
+                kBitsSmem, st, a, b, n_frames, y0 * kFB, kstride_bytes, op_a, op_b, s_a, s_b, chunks_a)) != cudaSuccess)
+                return e;
         }
         return cudaSuccess;
     }
@@ -425,10 +451,9 @@ cudaError_t launch_ingest(bool bf16, const FramesDev& a, const FramesDev& b, int
             FramesDev a2 = a, b2 = b;
             a2.data = a.data + t0 * kX4Frames * a.frame_stride;
             b2.data = b.data + t0 * kX4Frames * b.frame_stride;
-            ingest_u8x4_kernel<<<dim3((unsigned)(xa + xb), (unsigned)nt), 256, 0, st>>>(
-                a2, b2, n_frames - t0 * kX4Frames, kstride_bytes, op_a + t0 * kIngestRowBytes,
-                op_b + t0 * kIngestRowBytes, s_a, s_b, xa, vmax);
-            cudaError_t e = cudaGetLastError();
+            const cudaError_t e = launch_kernel(
+                zeroed, ingest_u8x4_kernel, dim3((unsigned)(xa + xb), (unsigned)nt), 256, 0, st, a2, b2,
+                n_frames - t0 * kX4Frames, kstride_bytes, op_a + t0 * kIngestRowBytes, op_b + t0 * kIngestRowBytes, s_a, s_b, xa, vmax);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;

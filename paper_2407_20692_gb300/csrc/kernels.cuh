@@ -10,6 +10,25 @@
 
 namespace cpi {
 
+// Launch of a kernel that begins with dep_wait() (ptx.cuh).  chain: its placement and
+// set-up overlap the end of the kernel before it in the stream, which must be one of
+// the same call (the first kernel of a call is launched plainly, after everything
+// its stream waits for). 
+template <typename... P, typename... A>
+cudaError_t launch_kernel(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chain ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Status bits recorded by kernels in the per-device status word.
 constexpr unsigned int kStatusTimeoutBit = 1u;
 
@@ -29,10 +48,10 @@ constexpr int kIngestRowBytes = 256;              // BF16 operand bytes per pixe
 inline int ingest_frames_per_cta(bool bf16) { return bf16 ? 128 : 256; }
 
 // vmax (BF16 path, may be null): the largest A and B value seen is raised into
-// vmax[0] and vmax[1] (the caller zeroes them first).
+// vmax[0] and vmax[1].  Both are zeroed first, and with zero_sums s_a and s_b too.
 cudaError_t launch_ingest(bool bf16, const FramesDev& a, const FramesDev& b, int64_t n_frames,
                           int64_t kstride_bytes, uint8_t* op_a, uint8_t* op_b, int64_t* s_a,
-                          int64_t* s_b, uint32_t* vmax, cudaStream_t st);
+                          int64_t* s_b, uint32_t* vmax, bool zero_sums, cudaStream_t st);
 
 // ------------------------------------------------------------------ moments
 // One raw-moment problem: S_ab of one (A, B) pair, split into work units of
@@ -73,7 +92,8 @@ struct MomentsShape {
 // block_n: the output tile's width, 256 (single correlations) or 128.
 MomentsShape moments_shape(bool bf16, int block_n = 256);
 
-cudaError_t launch_moments(bool bf16, int block_n, const MomentsLaunch<1>& L, int sm_count, cudaStream_t st);
+// chain (here and below): see launch_kernel
+cudaError_t launch_moments(bool bf16, int block_n, const MomentsLaunch<1>& L, int sm_count, bool chain, cudaStream_t st);
 cudaError_t launch_moments_group(bool bf16, int block_n, const MomentsLaunch<kMaxGroup>& L, int sm_count,
                                  cudaStream_t st);
 
@@ -81,7 +101,7 @@ cudaError_t launch_moments_group(bool bf16, int block_n, const MomentsLaunch<kMa
 cudaError_t launch_fold(const int32_t* partial, int n_chunks, int64_t M, int64_t N,
                         int64_t* s_ab, int accumulate, int write_sab, const int64_t* s_a,
                         const int64_t* s_b, int64_t n_frames, double* gamma, float* gamma_f32,
-                        cudaStream_t st, int wide = 0);
+                        cudaStream_t st, bool chain, int wide = 0);
 // wide != 0: the numerator N S_ab - S_a S_b is formed in 128 bits (sums from
 // accumulating calls, which the per-call overflow check does not bound).
 

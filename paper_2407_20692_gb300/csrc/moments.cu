@@ -155,8 +155,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     moments_kernel(const __grid_constant__ MomentsLaunch<K> L) {
     using C = MomentsCfg<kBf16, kBN>;
     __shared__ int seg_kb[K];   // BF16: K blocks per exact FP32 segment, per problem
-    if constexpr (kBf16)
-        for (int p = threadIdx.x; p < L.n_problems; p += blockDim.x) seg_kb[p] = segment_kblocks(L.prob[p]);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                ~static_cast<uintptr_t>(1023));
@@ -196,6 +194,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_alloc(tmem_slot, C::kTmemCols);
         tmem_relinquish();
     }
+    dep_wait();
+    dep_launch();
+    if constexpr (kBf16)
+        for (int p = threadIdx.x; p < L.n_problems; p += blockDim.x) seg_kb[p] = segment_kblocks(L.prob[p]);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -419,7 +421,7 @@ MomentsShape moments_shape(bool bf16, int block_n) {
 }
 
 template <bool kBf16, int kBN, int K>
-static cudaError_t launch_impl(const MomentsLaunch<K>& L, int sm_count, cudaStream_t st) {
+static cudaError_t launch_impl(const MomentsLaunch<K>& L, int sm_count, bool chain, cudaStream_t st) {
     // The shared-memory opt-in is a per-device function attribute: set it once per device.
     static bool attr_set[64] = {};
     int dev = 0;
@@ -434,26 +436,25 @@ static cudaError_t launch_impl(const MomentsLaunch<K>& L, int sm_count, cudaStre
         attr_set[dev] = true;
     }
     const int grid = L.n_units < sm_count ? L.n_units : sm_count;
-    moments_kernel<kBf16, kBN, K><<<grid, kThreads, C::kSmem, st>>>(L);
-    return cudaGetLastError();
+    return launch_kernel(chain, moments_kernel<kBf16, kBN, K>, grid, kThreads, C::kSmem, st, L);
 }
 
 template <int K>
-static cudaError_t launch_any(bool bf16, int block_n, const MomentsLaunch<K>& L, int sm_count, cudaStream_t st) {
+static cudaError_t launch_any(bool bf16, int block_n, const MomentsLaunch<K>& L, int sm_count, bool chain, cudaStream_t st) {
     if (block_n == 128)
-        return bf16 ? launch_impl<true, 128, K>(L, sm_count, st) : launch_impl<false, 128, K>(L, sm_count, st);
+        return bf16 ? launch_impl<true, 128, K>(L, sm_count, chain, st) : launch_impl<false, 128, K>(L, sm_count, chain, st);
     if (block_n == 256)
-        return bf16 ? launch_impl<true, 256, K>(L, sm_count, st) : launch_impl<false, 256, K>(L, sm_count, st);
+        return bf16 ? launch_impl<true, 256, K>(L, sm_count, chain, st) : launch_impl<false, 256, K>(L, sm_count, chain, st);
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_moments(bool bf16, int block_n, const MomentsLaunch<1>& L, int sm_count, cudaStream_t st) {
-    return launch_any<1>(bf16, block_n, L, sm_count, st);
+cudaError_t launch_moments(bool bf16, int block_n, const MomentsLaunch<1>& L, int sm_count, bool chain, cudaStream_t st) {
+    return launch_any<1>(bf16, block_n, L, sm_count, chain, st);
 }
 
 cudaError_t launch_moments_group(bool bf16, int block_n, const MomentsLaunch<kMaxGroup>& L, int sm_count,
                                  cudaStream_t st) {
-    return launch_any<kMaxGroup>(bf16, block_n, L, sm_count, st);
+    return launch_any<kMaxGroup>(bf16, block_n, L, sm_count, false, st);
 }
 
 }  // namespace cpi

@@ -18,6 +18,15 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
     return t;
 }
 
+// ---------------------------------------------------------------- programmatic launch
+// A kernel launched in a chain (launch_kernel) may start while the kernel before it in
+// the stream is finishing: dep_wait() returns once that kernel is complete and its
+// writes are visible.  Every thread calls it before its first access to memory that
+// another kernel reads or writes.  dep_launch() lets the next kernel's CTAs be
+// placed as soon as every CTA of this one has started (they wait in dep_wait()).
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- packed FP32
 // Two FP32 lanes in one 64-bit register pair, for the packed f32x2 instructions
 // of sm_100+ (each lane is an ordinary IEEE round-to-nearest FP32 operation).

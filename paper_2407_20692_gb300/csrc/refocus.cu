@@ -126,6 +126,8 @@ struct BandGeom {
 __global__ void __launch_bounds__(256) refocus_xtables_kernel(const PlaneBlock pl, int n_planes, int wa, int wb,
                                                               int pad_l, long long* __restrict__ xcol,
                                                               long long* __restrict__ xang) {
+    dep_wait();
+    dep_launch();
     const double cxa = 0.5 * (double)(wa - 1), cxb = 0.5 * (double)(wb - 1);
     const double sx = (double)wa / (double)wb;
     const long long bias = 128ll + ((long long)pad_l << 32);
@@ -186,6 +188,8 @@ __global__ void __launch_bounds__(kBandThreads, 1) refocus_band_kernel(const __g
         }
         fence_barrier_init();
     }
+    dep_wait();
+    dep_launch();
     __syncthreads();
     if (tid == 0)
         for (uint32_t q = 0; q < (uint32_t)stages && q < total_sl; ++q) issue(q);
@@ -354,6 +358,8 @@ struct RowGeom {
 // [slice][group][wa + 4][4] from [slice][ha][wa], zero columns and rows beyond the slice.
 __global__ void __launch_bounds__(256) refocus_interleave_kernel(const float* __restrict__ src, float4* __restrict__ dst,
                                                                  int64_t n, int ha, int wa, int groups) {
+    dep_wait();
+    dep_launch();
     const int XP = wa + 4;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t sg = i / XP;
@@ -428,6 +434,8 @@ __global__ void __launch_bounds__(kBandThreads, 1) refocus_rows_kernel(const flo
         }
         fence_barrier_init();
     }
+    dep_wait();
+    dep_launch();
     for (int p = tid; p < g.n_planes + PT; p += blockDim.x) step[p] = p < g.n_planes ? __ldg(g.xang + 2 * p + 1) : 0ll;
     __syncthreads();
     if (tid == 0)
@@ -591,6 +599,7 @@ struct YGeom {
 __global__ void __launch_bounds__(kYThreads) refocus_ystage_kernel(const float* __restrict__ ubuf, const YGeom g,
                                                                    const PlaneBlock pl, float* __restrict__ out) {
     extern __shared__ __align__(16) YTap ytab[];     // [RB][hb]
+    dep_launch();
     const int ha = g.ha, wa = g.wa, hb = g.hb, RB = g.RB;
     const int p = blockIdx.y;
     const int r0 = blockIdx.x * RB;
@@ -602,6 +611,7 @@ __global__ void __launch_bounds__(kYThreads) refocus_ystage_kernel(const float* 
         const long long uy = fix32(al * ((double)(r0 + rr) - cya) + cya) + fix32((be * sy) * ((double)br - cyb));
         ytab[i] = y_tap(uy, ha, wa);
     }
+    dep_wait();      // the taps depend on nothing: formed while the x stage ends
     __syncthreads();
     const int64_t Ma = (int64_t)ha * wa;
     const float* src = ubuf + (int64_t)p * hb * Ma;
@@ -654,6 +664,8 @@ __global__ void __launch_bounds__(kYThreads) refocus_ystage_kernel(const float* 
 // rows padded to a multiple of 4 (2-D staging) or 16 floats (3-D staging).
 __global__ void __launch_bounds__(256) refocus_repack_kernel(const float* __restrict__ src, float* __restrict__ dst,
                                                              int64_t rows, int wa, int pitch) {
+    dep_wait();
+    dep_launch();
     const int64_t n = rows * pitch;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = i / pitch;
@@ -744,8 +756,7 @@ cudaError_t launch_band_t(const CUtensorMap* tm, const BandGeom& g, const PlaneB
     auto kern = refocus_band_kernel<WS, KR, PT>;
     cudaError_t e = set_smem_attr(kern, slot, kSmemCap);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kBandThreads, smem, st>>>(*tm, g, pl, ubuf);
-    return cudaGetLastError();
+    return launch_kernel(true, kern, grid, kBandThreads, smem, st, *tm, g, pl, ubuf);
 }
 
 cudaError_t launch_band(const BandPlan& b, const CUtensorMap* tm, const BandGeom& g, const PlaneBlock& pl,
@@ -886,9 +897,9 @@ cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, 
         const int64_t n = Mb * rw.groups * (wa + 4);
         int64_t blocks = (n + 255) / 256;
         if (blocks > 16 * (int64_t)sm_count) blocks = 16 * (int64_t)sm_count;
-        refocus_interleave_kernel<<<(unsigned)blocks, 256, 0, st>>>(gamma_f32, reinterpret_cast<float4*>(copy), n, ha, wa,
-                                                                    rw.groups);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_kernel(false, refocus_interleave_kernel, (unsigned)blocks, 256, 0, st, gamma_f32,
+                                reinterpret_cast<float4*>(copy), n, ha, wa, rw.groups)) != cudaSuccess)
+            return e;
         gi = copy;
     } else {
         const float* src = gamma_f32;
@@ -898,8 +909,9 @@ cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, 
             const int64_t rows = Mb * ha;
             int64_t blocks = (rows * b.pitch + 255) / 256;
             if (blocks > 8 * (int64_t)sm_count) blocks = 8 * (int64_t)sm_count;
-            refocus_repack_kernel<<<(unsigned)blocks, 256, 0, st>>>(gamma_f32, copy, rows, wa, b.pitch);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if ((e = launch_kernel(false, refocus_repack_kernel, (unsigned)blocks, 256, 0, st, gamma_f32, copy, rows,
+                wa, b.pitch)) != cudaSuccess)
+                return e;
             src = copy;
             pitch = b.pitch;
         }
@@ -925,9 +937,10 @@ cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, 
             pb.alpha[i] = alpha[p0 + i];
             pb.beta[i] = beta[p0 + i];
         }
-        refocus_xtables_kernel<<<(unsigned)((np * kBandThreads + 255) / 256), 256, 0, st>>>(
-            pb, np, wa, wb, rw.ok ? 2 : b.pad_l, xcol, xang);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_kernel(p0 > 0 || rw.ok || b.pitch != 0, refocus_xtables_kernel,
+            (unsigned)((np * kBandThreads + 255) / 256), 256, 0, st, pb, np, wa, wb, rw.ok ? 2 : b.pad_l, xcol,
+            xang)) != cudaSuccess)
+            return e;
         if (rw.ok) {
             RowGeom g{};
             g.ha = ha;
@@ -951,8 +964,7 @@ cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, 
             const int64_t ctas = (int64_t)sm_count * rw.per_sm;
             const int grid = (int)(units < ctas ? units : ctas);
             if ((e = set_smem_attr(refocus_rows_kernel<8, 4>, 10, kSmemCap)) != cudaSuccess) return e;
-            refocus_rows_kernel<8, 4><<<grid, rw.threads, rw.smem, st>>>(gi, g, ubuf);
-            e = cudaGetLastError();
+            e = launch_kernel(true, refocus_rows_kernel<8, 4>, grid, rw.threads, rw.smem, st, gi, g, ubuf);
         } else {
             BandGeom g{};
             g.ha = ha;
@@ -981,9 +993,9 @@ cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, 
         YGeom y{ha, wa, hb, RB, p0};
         const size_t ysmem = (size_t)RB * hb * sizeof(YTap);
         if ((e = set_smem_attr(refocus_ystage_kernel, 20, kSmemCap)) != cudaSuccess) return e;
-        refocus_ystage_kernel<<<dim3((unsigned)((ha + RB - 1) / RB), (unsigned)np), kYThreads, ysmem, st>>>(ubuf, y, pb,
-                                                                                                           out);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_kernel(true, refocus_ystage_kernel, dim3((unsigned)((ha + RB - 1) / RB), (unsigned)np),
+            kYThreads, ysmem, st, ubuf, y, pb, out)) != cudaSuccess)
+            return e;
     }
     return cudaSuccess;
 }
