@@ -83,20 +83,17 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// 2-D K-major operand [rows][kstride_bytes], 128B swizzle.  BF16: tile box = 64
-// elements (128 bytes) x box_rows.  Binary (E2M1 packed two per byte): box =
-// 128 elements (64 bytes in HBM) x box_rows, each 8-byte group of 16 elements
-// landing in 16 bytes of shared memory (128 bytes per box row, the layout the
-// tensor cores read 4-bit operands in).
+// 2-D K-major operand [rows][kstride_bytes], 128B swizzle: a tile box is 128 bytes
+// of a row (64 BF16 values, or 256 E2M1 values packed two per byte) x box_rows.
 bool make_operand_map(CUtensorMap* m, void* base, bool bf16, int64_t rows, int64_t kstride_bytes,
                       int box_rows) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)(bf16 ? kstride_bytes / 2 : kstride_bytes * 2), (cuuint64_t)rows};
+    cuuint64_t dims[2] = {(cuuint64_t)(bf16 ? kstride_bytes / 2 : kstride_bytes), (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)kstride_bytes};
-    cuuint32_t box[2] = {(cuuint32_t)(bf16 ? 64 : 128), (cuuint32_t)box_rows};
+    cuuint32_t box[2] = {(cuuint32_t)(bf16 ? 64 : 128), (cuuint32_t)box_rows};   // 128 bytes
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(m, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_16U4_ALIGN16B, 2,
+    CUresult r = enc(m, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 2,
                      base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -159,7 +156,7 @@ FramesDev to_dev(const cpi_frames* f) {
 
 // Execution plan of one correlation.
 struct CorrPlan {
-    bool bf16;                 // BF16 operands (any 8-bit input) or FP8 (both binary)
+    bool bf16;                 // BF16 operands (any 8-bit input) or E2M1 (both binary)
     int64_t Ma, Mb, n;
     int64_t kstride_bytes;     // operand row length in bytes (frames padded to the ingest tile;
                                // 2 bytes per frame BF16, half a byte E2M1)
@@ -195,16 +192,17 @@ cpi_status make_plan_tiles(const cpi_frames* a, const cpi_frames* b, int64_t n, 
     p.tiles_m = (int)((p.Ma + 127) / 128);
     p.tiles_n = (int)((p.Mb + p.block_n - 1) / p.block_n);
     const int max_kb_chunk = kChunkFrames / sh.k_per_block;
+    const int min_kb = p.bf16 ? 8 : 4;   // K blocks of the shortest chunk worth a unit of its own
     const int64_t tiles = (int64_t)p.tiles_m * p.tiles_n;
     int n_chunks = (p.k_blocks + max_kb_chunk - 1) / max_kb_chunk;
     if (split >= 1) {
-        const int max_by_len = p.k_blocks / 8 > 0 ? p.k_blocks / 8 : 1;
+        const int max_by_len = p.k_blocks / min_kb > 0 ? p.k_blocks / min_kb : 1;
         n_chunks = n_chunks * split < max_by_len ? n_chunks * split : (max_by_len > n_chunks ? max_by_len : n_chunks);
     } else if (tiles < sm_count) {
         // small outputs: split the frames further so every SM gets work, but keep
-        // each chunk at least 8 K blocks long
+        // each chunk at least min_kb K blocks long
         int want = (int)(sm_count / tiles);
-        int max_by_len = p.k_blocks / 8;
+        int max_by_len = p.k_blocks / min_kb;
         if (max_by_len < 1) max_by_len = 1;
         if (want > max_by_len) want = max_by_len;
         if (want > n_chunks) n_chunks = want;

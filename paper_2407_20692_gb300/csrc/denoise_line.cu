@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) dnf_conv_kernel(const DnFlat 
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA issuer (whole warp, one lane issues)
-        constexpr uint32_t idesc = idesc_f32acc<true>(128, NOUT);
+        constexpr uint32_t idesc = idesc_bf16(128, NOUT);
         const uint32_t on = elect_one() ? 1u : 0u;
         bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(wbar, 0, abort_flag, status, timeout_ns)), any = false;
         const uint64_t bd0 = sdesc_plain(smem_u32(sw), NOUT * 16, 128);
@@ -380,13 +380,13 @@ __global__ void __launch_bounds__(kConvThreads, 1) dnf_conv_kernel(const DnFlat 
                     const uint64_t ad = ad0 + (uint64_t)(uint32_t)(tap / 3 * g.bstride + tap % 3 + t * 128);
 #pragma unroll
                     for (int h = 0; h < KC / 2; ++h)
-                        umma_f32_warp<true>(on, d, ad + (uint64_t)(2u * h * (uint32_t)g.SP),
+                        umma_bf16(on, d, ad + (uint64_t)(2u * h * (uint32_t)g.SP),
                                        bd0 + (uint64_t)((tap * KW + 2 * h % KW) * NOUT), idesc, (tap | h) ? 1u : 0u);
                 }
             }
             any = true;
-            umma_commit_warp(on, &empty[s]);
-            umma_commit_warp(on, &tfull[acc]);
+            umma_commit(on, &empty[s]);
+            umma_commit(on, &tfull[acc]);
             if (++s == stages) {
                 s = 0;
                 phase ^= 1;
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) dnf_conv_kernel(const DnFlat 
             }
         }
         if (!ok && any) {   // the MMAs issued must finish before the tensor memory is freed
-            umma_commit_warp(on, drain);
+            umma_commit(on, drain);
             mbar_wait_bounded(drain, 0, nullptr, nullptr, timeout_ns);
         }
     } else {
@@ -897,7 +897,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
                 mbar_wait_bounded(&full[j % (uint32_t)stages], (j / (uint32_t)stages) & 1u, nullptr, nullptr, a.timeout_ns);
     } else if (warp == 5) {
         // both operands MN-major
-        constexpr uint32_t idesc = idesc_f32acc<true>(128, NB) | (1u << 15) | (1u << 16);
+        constexpr uint32_t idesc = idesc_bf16(128, NB) | (1u << 15) | (1u << 16);
         const int64_t q16 = ((int64_t)g.Q + 15) / 16 * 16;      // delta and the input's margin are defined up to here
         const uint32_t on = elect_one() ? 1u : 0u;
         bool ok = true, any = false;
@@ -919,24 +919,24 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
             for (int k = 0; k < steps; ++k, ad += 16, bd += 16) {
 #pragma unroll
                 for (int ky = 0; ky < 3; ++ky)
-                    umma_f32_warp<true>(on, d + (uint32_t)(ky * NB), ad + (uint64_t)(uint32_t)(ky * a.bstride), bd, idesc,
+                    umma_bf16(on, d + (uint32_t)(ky * NB), ad + (uint64_t)(uint32_t)(ky * a.bstride), bd, idesc,
                                    first && k == 0 ? 0u : 1u);
             }
             any = true;
-            umma_commit_warp(on, &empty[s]);
+            umma_commit(on, &empty[s]);
             if (++s == stages) {
                 s = 0;
                 phase ^= 1;
             }
             if (!last) continue;
-            umma_commit_warp(on, &tfull[acc]);
+            umma_commit(on, &tfull[acc]);
             if (++acc == 2) {
                 acc = 0;
                 acc_phase ^= 1;
             }
         }
         if (!ok && any) {   // the MMAs issued must finish before the tensor memory is freed
-            umma_commit_warp(on, drain);
+            umma_commit(on, drain);
             mbar_wait_bounded(drain, 0, nullptr, nullptr, a.timeout_ns);
         }
     } else if (warp < kDrainWarps) {

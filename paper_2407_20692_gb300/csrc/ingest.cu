@@ -12,10 +12,8 @@
 //   - any other frames -> BF16 (1-bit frames that do not meet the first case as
 //     packed E2M1), one CTA per tile of 32 pixels x 128 (BF16) or 256 (E2M1)
 //     frames.
-// The raw-moment GEMM loads the packed E2M1 rows with a tensor map of 16 x 4-bit
-// groups, which spreads each 8-byte group over 16 bytes of shared memory: the
-// layout tcgen05 kind::f8f6f4 reads 4-bit operands in.  A binary operand row is
-// so half as many bytes in HBM and L2 as an 8-bit one would be.
+// The raw-moment GEMM reads the packed E2M1 rows as they stand (tcgen05 kind::mxf4):
+// a binary operand row is half as many bytes as an 8-bit one would be.
 // Frames at or beyond n_frames are written as 0, so every operand row is padded
 // to a whole number of CTA tiles.  The same pass adds the marginal sums
 // S_a = sum_i A_i (Eq. (1), second term) with exact int64 atomics.
@@ -453,7 +451,8 @@ cudaError_t launch_ingest(bool bf16, const FramesDev& a, const FramesDev& b, int
             b2.data = b.data + t0 * kX4Frames * b.frame_stride;
             const cudaError_t e = launch_kernel(
                 zeroed, ingest_u8x4_kernel, dim3((unsigned)(xa + xb), (unsigned)nt), 256, 0, st, a2, b2,
-                n_frames - t0 * kX4Frames, kstride_bytes, op_a + t0 * kIngestRowBytes, op_b + t0 * kIngestRowBytes, s_a, s_b, xa, vmax);
+                n_frames - t0 * kX4Frames, kstride_bytes, op_a + t0 * kIngestRowBytes, op_b + t0 * kIngestRowBytes, s_a,
+                s_b, xa, vmax);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;

@@ -2,9 +2,9 @@
 // first term of Eq. (1)) on the 5th-generation tensor cores.
 //
 // Operands are the K-major rows written by the ingest step (one row per pixel,
-// K = frames): E2M1 0/1 values for binary frames (tcgen05 kind::f8f6f4, packed
-// two per byte in HBM and spread to 16-byte groups in shared memory by TMA), or
-// BF16 integers 0..255 (kind::f16).  Products are small integers, accumulated
+// K = frames): E2M1 0/1 values for binary frames (packed two per byte, tcgen05
+// kind::mxf4 with every block scale 1.0: K = 64 per MMA), or BF16 integers 0..255
+// (kind::f16, K = 16).  Products are small integers, accumulated
 // in FP32 in tensor memory; a sum of integers stays exact while it is below
 // 2^24, and the schedule guarantees that:
 //   - binary frames: a frame chunk has at most 65536 frames, so every sum is
@@ -56,18 +56,19 @@ template <bool kBf16, int kBN>
 struct MomentsCfg {
     static constexpr int kBlockN = kBN;                         // 256 or 128 (batches tune it)
     static constexpr int kStages = kBN == 256 ? 4 : 6;
-    static constexpr int kElem = kBf16 ? 2 : 1;
-    static constexpr int kKPerBlock = kRowBytes / kElem;     // 64 / 128 elements
+    static constexpr int kKPerBlock = kBf16 ? kRowBytes / 2 : kRowBytes * 2;   // 64 / 256 elements
     static constexpr int kABytes = kBlockM * kRowBytes;       // 16 KiB
     static constexpr int kBBytes = kBlockN * kRowBytes;       // 32 KiB
-    // bytes a stage's copies deliver: E2M1 rows are 64 bytes in HBM, spread over
-    // the 128-byte shared-memory row (8 bytes of values per 16-byte group)
-    static constexpr uint32_t kTxBytes = kBf16 ? kABytes + kBBytes : (kABytes + kBBytes) / 2;
-    // tensor memory (2 x kBN columns): two FP32 accumulators, so the epilogue of
-    // one unit (FP8) or segment (BF16) overlaps the MMAs of the next; the BF16
-    // int32 running sums live in the epilogue threads' registers
-    static constexpr int kAcc = 2;
-    static constexpr uint32_t kTmemCols = 2 * kBN;
+    static constexpr uint32_t kTxBytes = kABytes + kBBytes;
+    // tensor memory: FP32 accumulators, two where they fit, so that the epilogue of
+    // one unit (E2M1) or segment (BF16) overlaps the MMAs of the next; the BF16
+    // running sums live in the epilogue threads' registers.  E2M1: behind them 32
+    // columns of block scales, every byte 127 (2^0 in UE8M0), which leaves room for
+    // one accumulator of 256 columns; its epilogue takes the whole tile into
+    // registers and hands it back before it converts and stores.
+    static constexpr int kSfCols = kBf16 ? 0 : 32;
+    static constexpr int kAcc = 2 * kBN + kSfCols <= 512 ? 2 : 1;
+    static constexpr uint32_t kTmemCols = kAcc * kBN + kSfCols > 256 ? 512 : 256;
     static constexpr size_t kSmem = 1024 + (size_t)kStages * (kABytes + kBBytes) + 256;
 };
 
@@ -202,10 +203,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    const uint32_t sf = tmem_base + (uint32_t)(C::kAcc * C::kBlockN);   // E2M1: block scales
+    if constexpr (!kBf16) {
+        if (warp >= 2 && warp < 6) tmem_fill_32x32b_x32(sf + ((uint32_t)(32 * (warp & 3)) << 16), 0x7F7F7F7Fu);
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+    }
 
     if (warp == 0) {
         if (lane == 0) {
             // ---------------------------------------------------------- producer
+            constexpr int kBoxX = kBf16 ? kRowBytes / 2 : kRowBytes;   // map elements per K block (BF16 / bytes)
             int stage = 0;
             uint32_t phase = 0;
             uint32_t issued_mask = 0, issued_phase = 0;   // per stage: loaded at least once / parity
@@ -220,10 +229,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                         break;
                     }
                     mbar_arrive_expect_tx(&full[stage], C::kTxBytes);
-                    tma_load_2d(sA + stage * C::kABytes, ma, &full[stage], kb * C::kKPerBlock,
-                                w.tm * kBlockM);
-                    tma_load_2d(sB + stage * C::kBBytes, mb, &full[stage], kb * C::kKPerBlock,
-                                w.tn * C::kBlockN);
+                    tma_load_2d(sA + stage * C::kABytes, ma, &full[stage], kb * kBoxX, w.tm * kBlockM);
+                    tma_load_2d(sB + stage * C::kBBytes, mb, &full[stage], kb * kBoxX, w.tn * C::kBlockN);
                     issued_mask |= 1u << stage;
                     issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
                     if (++stage == C::kStages) {
@@ -245,12 +252,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---------------------------------------------------------- MMA issuer
             // The whole warp runs the loop and one lane issues: the descriptors
             // stay in uniform registers.
-            // The tensor pipe takes one 128 x 256 x 16 (BF16) or x 32 (E2M1) MMA
+            // The tensor pipe takes one 128 x 256 x 16 (BF16) or x 64 (E2M1) MMA
             // per 128 cycles only while this thread issues the next one within
             // that time, so the loop keeps its per-K-block work to a few adds:
             // segment bounds are counted down (no division), descriptors step
             // by the stage size.
-            constexpr uint32_t idesc = idesc_f32acc<kBf16>(kBlockM, C::kBlockN);
+            constexpr uint32_t idesc =
+                kBf16 ? idesc_bf16(kBlockM, C::kBlockN) : idesc_mxf4(kBlockM, C::kBlockN);
             const uint64_t da0 = sdesc_kmajor_sw128(smem_u32(sA));
             const uint64_t db0 = sdesc_kmajor_sw128(smem_u32(sB));
             const uint32_t on = elect_one() ? 1u : 0u;
@@ -268,17 +276,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const bool seg_start = seg_left == 0;
                     if (seg_start) {
                         seg_left = min(kb_per_seg, nkb - i);
-                        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, status, tmo))) {
-                            ok = false;
-                            break;
-                        }
+                        ok = __all_sync(0xffffffffu,
+                                        mbar_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, status, tmo));
+                        if (!ok) break;
                         tc_fence_after();
                     }
                     --seg_left;
-                    if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[stage], phase, abort_flag, status, tmo))) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[stage], phase, abort_flag, status, tmo));
+                    if (!ok) break;
                     tc_fence_after();
                     const uint32_t d = tmem_base + (uint32_t)(acc * C::kBlockN);
                     const uint64_t da = da0 + (uint64_t)(stage * (C::kABytes >> 4));
@@ -286,17 +291,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                     for (int k = 0; k < kRowBytes / 32; ++k) {
                         // advance the start address by 32 bytes (2 x 16-byte units) per MMA
-                        umma_f32_warp<kBf16>(on, d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc,
-                                             (seg_start && k == 0) ? 0u : 1u);
+                        const uint32_t add = seg_start && k == 0 ? 0u : 1u;
+                        if constexpr (kBf16)
+                            umma_bf16(on, d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, add);
+                        else
+                            umma_mxf4(on, d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, sf, sf, add);
                     }
                     issued_any = true;
-                    umma_commit_warp(on, &empty[stage]);
+                    umma_commit(on, &empty[stage]);
                     if (++stage == C::kStages) {
                         stage = 0;
                         phase ^= 1;
                     }
                     if (seg_left == 0) {   // segment (BF16) or unit (E2M1) done: hand the accumulator over
-                        umma_commit_warp(on, &tfull[acc]);
+                        umma_commit(on, &tfull[acc]);
                         if (++acc == C::kAcc) {
                             acc = 0;
                             acc_phase ^= 1;
@@ -305,7 +313,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
             if (!ok && issued_any) {
-                umma_commit_warp(on, drain);
+                umma_commit(on, drain);
                 mbar_wait_bounded(drain, 0, nullptr, nullptr, tmo);
             }
         }
@@ -335,18 +343,20 @@ __global__ void __launch_bounds__(kThreads, 1)
                     break;
                 }
                 tc_fence_after();
-#pragma unroll 1
-                for (int c = 0; c < kHalf / 32; ++c) {
-                    uint32_t r[32];
-                    tmem_ld_32x32b_x32(tmem_base + lane_addr + (uint32_t)(acc * C::kBlockN) + col0 + c * 32, r);
-                    tmem_ld_wait();
-                    int32_t v[32];
+                uint32_t r[kHalf / 32][32];
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = __float2int_rn(__uint_as_float(r[j]));
-                    store_row_chunk(P, chunk, m, n0 + c * 32, v);
-                }
+                for (int c = 0; c < kHalf / 32; ++c)
+                    tmem_ld_32x32b_x32(tmem_base + lane_addr + (uint32_t)(acc * C::kBlockN) + col0 + c * 32, r[c]);
+                tmem_ld_wait();
                 tc_fence_before();
                 mbar_arrive(&tempty[acc]);
+#pragma unroll
+                for (int c = 0; c < kHalf / 32; ++c) {
+                    int32_t v[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = __float2int_rn(__uint_as_float(r[c][j]));
+                    store_row_chunk(P, chunk, m, n0 + c * 32, v);
+                }
                 if (++acc == C::kAcc) {
                     acc = 0;
                     acc_phase ^= 1;

@@ -217,34 +217,20 @@ __device__ __forceinline__ uint64_t sdesc_kmajor_sw128(uint32_t saddr) {
     return d;
 }
 
-// Instruction descriptor: D = F32, A and B K-major, shape M x N.
-// kBf16: kind::f16 with BF16 operands (format 1); else kind::f8f6f4 with E2M1
-// operands (format 5: 4-bit values, 16 per 16-byte shared-memory group).
-template <bool kBf16>
-__host__ __device__ constexpr uint32_t idesc_f32acc(int M, int N) {
+// Instruction descriptors: D = F32, A and B K-major, shape M x N.
+// kind::f16 with BF16 operands (format 1).
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4)                                    // D format F32
-           | ((kBf16 ? 1u : 5u) << 7)                   // A format: BF16 (1) / E2M1 (5)
-           | ((kBf16 ? 1u : 5u) << 10)                  // B format
+           | (1u << 7) | (1u << 10)                     // A, B format BF16
            | ((uint32_t)(N >> 3) << 17)                 // N / 8
            | ((uint32_t)(M >> 4) << 24);                // M / 16
 }
-
-template <bool kBf16>
-__device__ __forceinline__ void umma_f32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-    if constexpr (kBf16) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
-    }
+// kind::mxf4 (dense, K = 64): E2M1 operands (format 1), scale factors UE8M0.
+__host__ __device__ constexpr uint32_t idesc_mxf4(int M, int N) {
+    return (1u << 7) | (1u << 10)                       // A, B format E2M1
+           | ((uint32_t)(N >> 3) << 17)                 // N / 8
+           | (1u << 23)                                 // scale format UE8M0
+           | ((uint32_t)(M >> 4) << 24);                // M / 16
 }
 
 // One lane of a converged warp (the same one each time).
@@ -254,28 +240,30 @@ __device__ __forceinline__ bool elect_one() {
     return e != 0;
 }
 
-// umma_f32 and umma_commit for a whole converged warp of which only the lane with
+// The MMA and its commit for a whole converged warp of which only the lane with
 // `on` != 0 issues: the operands stay warp-uniform, so they need no move from one
-// lane's registers into the uniform registers the instruction reads (which, per
-// MMA, costs more than a small tile's multiplication).
-template <bool kBf16>
-__device__ __forceinline__ void umma_f32_warp(uint32_t on, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                              uint32_t accumulate) {
-    if constexpr (kBf16) {
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-            "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(on)
-            : "memory");
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-            "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(on)
-            : "memory");
-    }
+// lane's registers into the uniform registers the instruction reads (measured: a
+// single diverged lane issues one MMA per 75 to 80 cycles whatever its size).
+__device__ __forceinline__ void umma_bf16(uint32_t on, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                          uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(on)
+        : "memory");
 }
-__device__ __forceinline__ void umma_commit_warp(uint32_t on, uint64_t* bar) {
+// Block-scaled 4-bit operands; scale factors (one per 32 elements of a row) in tensor
+// memory at sf_a and sf_b.
+__device__ __forceinline__ void umma_mxf4(uint32_t on, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                          uint32_t sf_a, uint32_t sf_b, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 q, %7, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%4], [%5], p;\n\t}" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(sf_a), "r"(sf_b), "r"(accumulate), "r"(on)
+        : "memory");
+}
+// Arrive on `bar` once every tcgen05 operation issued so far by the issuing lane is done.
+__device__ __forceinline__ void umma_commit(uint32_t on, uint64_t* bar) {
     asm volatile(
         "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
         "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)),
@@ -283,11 +271,12 @@ __device__ __forceinline__ void umma_commit_warp(uint32_t on, uint64_t* bar) {
         : "memory");
 }
 
-// Arrive on `bar` once every tcgen05 operation issued so far by this thread is done.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
+// v into 32 lanes x 32 consecutive 32-bit columns.
+__device__ __forceinline__ void tmem_fill_32x32b_x32(uint32_t taddr, uint32_t v) {
     asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_u32(bar))
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,"
+        "%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};\n\ttcgen05.wait::st.sync.aligned;" ::"r"(taddr),
+        "r"(v)
         : "memory");
 }
 
