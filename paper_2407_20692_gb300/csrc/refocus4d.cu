@@ -60,6 +60,8 @@ __device__ __forceinline__ void r4_kahan(float& acc, float& cmp, float v) {
 //   y axis: the same with rows (ha, hb, sy).
 __global__ void r4_tables_kernel(const Plane4Block co, int np, int ha, int wa, int hb, int wb,
                                  long long* __restrict__ t, int64_t stride) {
+    dep_wait();
+    dep_launch();
     const int p = blockIdx.x;
     if (p >= np) return;
     const double al = co.c[p][0], be = co.c[p][1], ga = co.c[p][2], de = co.c[p][3];
@@ -163,6 +165,8 @@ __global__ void __launch_bounds__(kColThreads, 1) r4_cols_kernel(const float* __
                        : 0.0f;
         BoxOf<K>::set(box[i], v);
     }
+    dep_launch();
+    dep_wait();   // Gamma was complete before the tables' kernel began
     for (int p0 = 0; p0 < np; p0 += G) {
         const int gp = min(G, np - p0);
         __syncthreads();   // boxes ready / previous pass's tables consumed
@@ -236,6 +240,8 @@ __global__ void __launch_bounds__(kColThreadsG) r4_cols_global_kernel(const floa
     const int64_t ma = (int64_t)ha * wa;
     longlong2* sB = reinterpret_cast<longlong2*>(sm);
     const float* gbase = g + ((int64_t)yb * wb) * ma + (int64_t)ya * wa;
+    dep_wait();
+    dep_launch();
     for (int p0 = 0; p0 < np; p0 += G) {
         const int gp = min(G, np - p0);
         __syncthreads();
@@ -299,6 +305,8 @@ __global__ void __launch_bounds__(kR4Threads) r4_rows_kernel(const float* __rest
                                                              int hb, const long long* __restrict__ t, int64_t stride,
                                                              float* __restrict__ out) {
     const int p = blockIdx.y;
+    dep_wait();
+    dep_launch();
     for (int w = threadIdx.x; w < G * wa; w += kR4Threads) {
         const int k = w / wa, xc = w - k * wa, xr = blockIdx.x * G + k;
         if (xr >= ha) continue;
@@ -406,8 +414,8 @@ cudaError_t launch_cols(const ColPlan& c, const float* g, int np, int ha, int wa
         attr[dev] = true;
     }
     const dim3 grid((unsigned)hb, (unsigned)((ha + K - 1) / K));
-    r4_cols_kernel<K><<<grid, c.threads, c.smem, st>>>(g, np, c.G, ha, wa, hb, wb, c.WP, t, stride, c_hi, c_lo);
-    return cudaGetLastError();
+    return launch_kernel(true, r4_cols_kernel<K>, grid, c.threads, c.smem, st, g, np, c.G, ha, wa, hb, wb, c.WP, t, stride,
+                         c_hi, c_lo);
 }
 }  // namespace
 
@@ -416,8 +424,7 @@ cudaError_t launch_refocus4d_chunk(const float* gamma_f32, int ha, int wa, int h
     long long* t = reinterpret_cast<long long*>(ws + L.tables);
     float* c_hi = reinterpret_cast<float*>(ws + L.c_hi);
     float* c_lo = reinterpret_cast<float*>(ws + L.c_lo);
-    r4_tables_kernel<<<np, 128, 0, st>>>(coef, np, ha, wa, hb, wb, t, L.stride);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(false, r4_tables_kernel, np, 128, 0, st, coef, np, ha, wa, hb, wb, t, L.stride);
     if (e != cudaSuccess) return e;
     double skew = 0.0;
     for (int p = 0; p < np; ++p) skew += (coef.c[p][0] - 1.0) * coef.c[p][2];
@@ -437,15 +444,13 @@ cudaError_t launch_refocus4d_chunk(const float* gamma_f32, int ha, int wa, int h
                 return e;
             attr[dev] = true;
         }
-        r4_cols_global_kernel<<<dim3((unsigned)hb, (unsigned)ha), kColThreadsG, sizeof(longlong2) * (size_t)G * wb, st>>>(
-            gamma_f32, np, G, ha, wa, hb, wb, t, L.stride, c_hi, c_lo);
-        e = cudaGetLastError();
+        e = launch_kernel(true, r4_cols_global_kernel, dim3((unsigned)hb, (unsigned)ha), kColThreadsG,
+                          sizeof(longlong2) * (size_t)G * wb, st, gamma_f32, np, G, ha, wa, hb, wb, t, L.stride, c_hi, c_lo);
     }
     if (e != cudaSuccess) return e;
     const int Gr = wa < kR4Threads ? kR4Threads / wa : 1;
-    r4_rows_kernel<<<dim3((unsigned)((ha + Gr - 1) / Gr), (unsigned)np), kR4Threads, 0, st>>>(c_hi, c_lo, Gr, ha, wa,
-                                                                                            hb, t, L.stride, out);
-    return cudaGetLastError();
+    return launch_kernel(true, r4_rows_kernel, dim3((unsigned)((ha + Gr - 1) / Gr), (unsigned)np), kR4Threads, 0, st,
+        c_hi, c_lo, Gr, ha, wa, hb, t, L.stride, out);
 }
 
 }  // namespace cpi
