@@ -25,6 +25,7 @@ namespace {
 
 constexpr int kMaxTiles = 4;                // 128-pixel tiles per unit
 constexpr int kLineRound = 1024;            // the longest unit of any pass (512 on the tensor cores)
+constexpr uint32_t kShortLine = 1u << 15;   // positions: below, units of one tile
 constexpr int kMaxStages = 4;
 constexpr int kConvThreads = 320;           // warp 0 copies, warp 1 issues MMAs, warps 2..9 epilogue
 constexpr int kEpiThreads = 256;
@@ -155,6 +156,7 @@ __global__ void __launch_bounds__(kStackThreads) dnf_stack_kernel(
     const Margins mg, int w_elems, __nv_bfloat16* __restrict__ wt) {
     dep_wait();
     dep_launch();
+    part = after_wait(part);
     if ((int)blockIdx.x >= stack_blocks) {
         const int i = ((int)blockIdx.x - stack_blocks) * kStackThreads + (int)threadIdx.x;
         if (i >= w_elems) return;
@@ -230,7 +232,7 @@ __global__ void __launch_bounds__(kStackThreads) dnf_stack_kernel(
 // pixels of the line.  Warp 0 (one thread) stages the weights once and then, per
 // unit, the line from one row above to one row below (the three bands of U + 2
 // pixels a row apart: one contiguous copy per plane, or three when a row is longer
-// than a unit); warp 1 (one thread) issues per tile of 128 pixels 9 taps x KC / 2
+// than a unit); warp 1 (one lane of it) issues per tile of 128 pixels 9 taps x KC / 2
 // MMAs (M = 128 pixels, N = NOUT channels, K = 16) into one of two TMEM
 // accumulators and frees the stage; warps 2..9 drain the other accumulator:
 //   kHidden: bias, ReLU, bf16, planes (zeros in the padding);
@@ -245,7 +247,10 @@ __global__ void __launch_bounds__(kStackThreads) dnf_stack_kernel(
 // and MMAs, frees its tensor memory and stops.
 //
 // What bounds it: an MMA of N = 32 is limited by reading A (128 x 16 bf16) from
-// shared memory, and a hidden layer moves 128 bytes per pixel through HBM.
+// shared memory (55 cycles each), and a hidden layer moves 128 bytes per pixel
+// through HBM (1024 slices of 64 x 64: 115 us, 0.50 GB at 4.3 TB/s; 175 us with the
+// MMAs issued by a diverged lane).  Units of 512 pixels, so that the row before and
+// after adds a quarter to what is staged; 8 epilogue warps drain two tiles at a time.
 enum Mode { kHidden, kInfer, kTrain, kGrad };
 
 struct ConvArgs {
@@ -405,7 +410,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) dnf_conv_kernel(const DnFlat 
         const int quarter = warp & 3;                             // TMEM lane quarter of this warp
         const int half = (warp - 2) >> 2;                         // tiles half, half + 2, ...
         const int64_t HW = (int64_t)g.H * g.W;
-        const float sc = kLast ? __ldg(a.scale) : 1.0f;
+        const float sc = kLast ? __ldg(after_wait(a.scale)) : 1.0f;
         int acc = 0;
         uint32_t acc_phase = 0;
         for (int u = blockIdx.x; u < g.n_units; u += gridDim.x) {
@@ -552,6 +557,7 @@ __global__ void __launch_bounds__(kExThreads, 2) dnf_conv_exact_kernel(const DnF
                                                                        const float* __restrict__ w) {
     dep_wait();
     dep_launch();
+    const uint8_t* const planes = after_wait(a.in);
     constexpr int U = ex_unit(COUT), KC = CIN == 9 ? 2 : 4;
     constexpr int WS = COUT == 1 ? 12 : 9 * COUT;               // weights per input channel
     extern __shared__ __align__(16) float sm_ex[];
@@ -566,7 +572,7 @@ __global__ void __launch_bounds__(kExThreads, 2) dnf_conv_exact_kernel(const DnF
     const int pxg = COUT == 1 ? warp : warp & 1, cog = COUT == 1 ? 0 : warp >> 1;
     const int base = pxg * (COUT == 1 ? 128 : 256) + lane * 4;
     const int64_t HW = (int64_t)g.H * g.W;
-    const float sc = MODE == kHidden ? 1.0f : __ldg(a.scale);
+    const float sc = MODE == kHidden ? 1.0f : __ldg(after_wait(a.scale));
     double lsum = 0.0;
     float bsum = 0.0f;
 
@@ -583,7 +589,7 @@ __global__ void __launch_bounds__(kExThreads, 2) dnf_conv_exact_kernel(const DnF
 #pragma unroll 1
         for (int c = 0; c < KC; ++c) {
             __syncthreads();                                    // the previous plane is consumed
-            const uint8_t* src = a.in + ((int64_t)c * g.PL + first) * 16;
+            const uint8_t* src = planes + ((int64_t)c * g.PL + first) * 16;
             for (int i = tid; i < g.SP; i += kExThreads) {
                 int64_t o = i;
                 if (g.Wp > U) {                                 // separate bands of bstride positions
@@ -719,6 +725,7 @@ __global__ void __launch_bounds__(kTopThreads) dnf_top_grad_kernel(const DnFlat 
                                                                    float* __restrict__ bias_part) {
     dep_wait();
     dep_launch();
+    rec = after_wait(rec);
     __shared__ __align__(16) float sw[9][32];
     __shared__ float bred[kTopThreads / 32][32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -798,13 +805,15 @@ __global__ void __launch_bounds__(kTopThreads) dnf_top_grad_kernel(const DnFlat 
 // (rows past 3 KC x 8 multiply whatever lies behind and are dropped); N = NB columns:
 // the hi and lo terms of delta (4 + 4 planes; the last layer: one plane of records,
 // columns 0..2); TMEM columns ky NB + n.  Warp 4 (one thread) copies, warp 5 (one
-// thread) issues, warps 0..3 add every unit's sums to FP32 registers while the next
+// lane of it) issues, warps 0..3 add every unit's sums to FP32 registers while the next
 // unit runs into the other accumulator: tensor-core sums are truncated, so an
 // accumulator left to grow over all of a CTA's pixels is biased in proportion to
 // their number (measured on the last layer, whose terms cancel: 7.4e-6 of the
 // gradient at 80x80 vs 12x12 against 4.6e-7 in FP32).  hold: images 64 wide, whose
-// gradients have always been summed that way, keep one accumulator to the end, so
-// that training there goes on as it was.  At the end the CTA writes rows (kx, ci) x
+// gradients have always been summed that way, keep one accumulator to the end over
+// the same blocks of up to 32 rows of a slice per CTA, so that training there goes
+// on as it was.  1024 slices of 64 x 64, 32 -> 32: 194 us, 0.83 GB at 4.3 TB/s.  At the
+// end the CTA writes rows (kx, ci) x
 // columns (ky, n) to part[cta].  Every wait is bounded.
 constexpr int kWgThreads = 192;
 constexpr int kWgMaxStages = 4;
@@ -813,11 +822,39 @@ struct WgArgs {
     const uint8_t* d_hi;        // NB = 64: 4 planes; NB = 16: the record plane
     const uint8_t* d_lo;
     float* part;
-    int U, n_units, bstride, SP, stages;
-    bool hold;                  // one accumulator for all units
+    int U, bstride, SP, stages;
+    int n_blocks;               // runs of pixels that CTAs take: U of them, or (hold) rows of one slice
+    bool hold;                  // one accumulator for all of a CTA's blocks
     uint32_t slack;             // bytes behind the ring that the dropped rows may touch
     unsigned int* status;
     unsigned long long timeout_ns;
+};
+
+// A CTA's way through its blocks, U pixels at a time.
+constexpr int kHoldRows = 32;
+struct WgWalk {
+    int v;               // block
+    int64_t q, left;     // first pixel, pixels of the block from there on (a multiple of 16)
+    __device__ __forceinline__ void block(const DnFlat& g, const WgArgs& a, int i) {
+        v = i;
+        if (v >= a.n_blocks) return;
+        if (a.hold) {   // the last rows of a slice may run on into its zero row
+            const int rows = min(g.H, kHoldRows), per = (g.H + rows - 1) / rows;
+            const int b = v / per, y0 = (v - b * per) * rows;
+            q = ((int64_t)b * (g.H + 1) + y0) * g.Wp;
+            left = ((int64_t)min(rows, g.H - y0) * g.Wp + 15) / 16 * 16;
+        } else {        // delta and the input's margin are defined up to the next multiple of 16
+            q = (int64_t)v * a.U;
+            left = min((int64_t)a.U, ((int64_t)g.Q + 15) / 16 * 16 - q);
+        }
+    }
+    __device__ __forceinline__ bool live(const WgArgs& a) const { return v < a.n_blocks; }
+    __device__ __forceinline__ bool last(const WgArgs& a) const { return left <= a.U && v + (int)gridDim.x >= a.n_blocks; }
+    __device__ __forceinline__ void next(const DnFlat& g, const WgArgs& a) {
+        q += a.U;
+        left -= a.U;
+        if (left <= 0) block(g, a, v + (int)gridDim.x);
+    }
 };
 
 template <int KC, int NB>
@@ -868,13 +905,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
     if (warp == 4 && lane == 0) {
         uint32_t k = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < a.n_units; u += gridDim.x, ++k) {
+        WgWalk w;
+        for (w.block(g, a, (int)blockIdx.x); w.live(a); w.next(g, a), ++k) {
             const int s = (int)(k % (uint32_t)stages);
             if (!mbar_wait_bounded(&empty[s], ((k / (uint32_t)stages) & 1u) ^ 1u, abort_flag, a.status, a.timeout_ns)) {
                 ok = false;
                 break;
             }
-            const int64_t at = (g.G + (int64_t)u * a.U) * 16;
+            const int64_t at = (g.G + w.q) * 16;
             uint8_t* dst = ring + (size_t)s * stage_bytes;
             mbar_arrive_expect_tx(&full[s], (NB == 64 ? 8u : 1u) * dplane + 3u * KC * aplane);
             for (int c = 0; c < (NB == 64 ? 8 : 1); ++c)
@@ -898,20 +936,19 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
     } else if (warp == 5) {
         // both operands MN-major
         constexpr uint32_t idesc = idesc_bf16(128, NB) | (1u << 15) | (1u << 16);
-        const int64_t q16 = ((int64_t)g.Q + 15) / 16 * 16;      // delta and the input's margin are defined up to here
         const uint32_t on = elect_one() ? 1u : 0u;
         bool ok = true, any = false;
         int s = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
-        for (int u = blockIdx.x; u < a.n_units; u += gridDim.x) {
-            const bool first = !a.hold || !any, last = !a.hold || u + (int)gridDim.x >= a.n_units;
+        WgWalk w;
+        for (w.block(g, a, (int)blockIdx.x); w.live(a); w.next(g, a)) {
+            const bool first = !a.hold || !any, last = !a.hold || w.last(a);
             ok = (!first || mbar_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, a.status, a.timeout_ns)) &&
                  mbar_wait_bounded(&full[s], phase, abort_flag, a.status, a.timeout_ns);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            const int64_t left = q16 - (int64_t)u * a.U;
-            const int steps = (int)(left < a.U ? left : a.U) / 16;
+            const int steps = (int)min(w.left, (int64_t)a.U) / 16;
             const uint32_t base = smem_u32(ring + (size_t)s * stage_bytes);
             const uint32_t d = tmem_base + (uint32_t)acc * kCols;
             uint64_t bd = sdesc_plain(base, 128, dplane);
@@ -946,7 +983,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
         bool ok = true;
         int acc = 0;
         uint32_t acc_phase = 0;
-        for (int u = blockIdx.x; u < a.n_units; u += a.hold ? a.n_units : (int)gridDim.x) {
+        for (int v = blockIdx.x; v < a.n_blocks; v += a.hold ? a.n_blocks : (int)gridDim.x) {
             if (!mbar_wait_bounded(&tfull[acc], acc_phase, abort_flag, a.status, a.timeout_ns)) {
                 ok = false;
                 break;
@@ -995,6 +1032,9 @@ __global__ void __launch_bounds__(256) dnf_wgrad_reduce_kernel(const float* __re
                                                                float* __restrict__ grad, float* __restrict__ loss) {
     dep_wait();
     dep_launch();
+    part = after_wait(part);
+    bias_part = after_wait(bias_part);
+    loss_part = after_wait(loss_part);
     constexpr int NB = COUT == 32 ? 64 : 16, kCols = 3 * NB, kRows = 3 * KC * 8;
     __shared__ float red[8][32];
     const int co = threadIdx.x & 31, grp = threadIdx.x >> 5;
@@ -1060,7 +1100,7 @@ constexpr size_t kDynMax = kSmemMax - 2048;      // the static sums of the train
 template <int KC, int NOUT>
 int choose_tiles(const DnFlat& g, int sm_count, size_t* fixed) {
     *fixed = 128 + (size_t)weight_elems(KC == 8 ? 4 : KC, NOUT) * 2 + 128;
-    int T = kMaxTiles;
+    int T = g.Q < kShortLine ? 1 : kMaxTiles;
     while (T > 1 && ((int64_t)g.Q + T * 128 - 1) / (T * 128) < 2 * (int64_t)sm_count) T /= 2;
     for (; T > 1; T /= 2) {
         const int U = T * 128;
@@ -1129,10 +1169,16 @@ cudaError_t launch_wgrad(const DnFlat& g, WgArgs a, const float* bias_part, int 
     size_t stage = shape(U);
     while (U > 64 && (256 + a.slack + 2 * stage > kDynMax || ((int64_t)g.Q + U - 1) / U < sm_count)) stage = shape(U -= 16);
     if (256 + a.slack + 2 * stage > kDynMax) return cudaErrorInvalidValue;
+    a.n_blocks = (int)(((int64_t)g.Q + U - 1) / U);
+    if (a.hold) {
+        const int rows = g.H < kHoldRows ? g.H : kHoldRows;
+        const int len = (rows * g.Wp + 15) / 16, parts = (16 * len + U - 1) / U;     // even parts of a block
+        stage = shape(U = (len + parts - 1) / parts * 16);
+        a.n_blocks = (int)((int64_t)g.Q / g.Wp / (g.H + 1)) * ((g.H + rows - 1) / rows);
+    }
     a.stages = (int)((kDynMax - 256 - a.slack) / stage);
     if (a.stages > kWgMaxStages) a.stages = kWgMaxStages;
-    a.n_units = (int)(((int64_t)g.Q + U - 1) / U);
-    int grid = a.n_units < sm_count ? a.n_units : sm_count;
+    int grid = a.n_blocks < sm_count ? a.n_blocks : sm_count;
     if (grid > kDnMaxCtas) grid = kDnMaxCtas;
     e = launch_kernel(in_chain(g), dnf_wgrad_kernel<KC, NB>, grid, kWgThreads, 256 + a.stages * stage + a.slack, st, g, a);
     if (e != cudaSuccess) return e;
@@ -1168,7 +1214,8 @@ bool dn_flat_plan(int ha, int wa, int hb, int wb, bool training, size_t ws_bytes
     if (Q >= ((int64_t)1 << 31) - kLineRound) return false;
     g.Q = (uint32_t)Q;
     g.G = g.Wp + 1;
-    const int round = g.tensor ? kLineRound / 2 : kLineRound;
+    // the longest unit of any pass (short lines on the tensor cores run in units of 128)
+    const int round = !g.tensor ? kLineRound : (Q < kShortLine ? 128 : kLineRound / 2);
     g.PL = g.G + (Q + round - 1) / round * round + g.Wp + 1;
     size_t o = 0;
     auto take = [&](size_t bytes) {

@@ -43,6 +43,9 @@ __global__ void __launch_bounds__(256, 4) fold_kernel(const int32_t* __restrict_
                                                    float* gamma_f32) {
     dep_wait();
     dep_launch();
+    partial = after_wait(partial);
+    s_a = after_wait(s_a);
+    s_b = after_wait(s_b);
     __shared__ float tile[kTile][kTile + 1];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;    // 32 x 8
     const Idx b = (Idx)blockIdx.x * kTile + tx;

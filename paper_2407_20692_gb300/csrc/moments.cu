@@ -144,7 +144,10 @@ __device__ __forceinline__ Unit decode_unit(const MomentsLaunch<K>& L, int u) {
 // 255 x 255 when they are missing).
 __device__ __forceinline__ int segment_kblocks(const MomentsProblem& P) {
     uint64_t prod = 255u * 255u;
-    if (P.vmax != nullptr) prod = (uint64_t)__ldcg(P.vmax) * (uint64_t)__ldcg(P.vmax + 1);
+    if (P.vmax != nullptr) {
+        const uint32_t* v = after_wait(P.vmax);
+        prod = (uint64_t)__ldcg(v) * (uint64_t)__ldcg(v + 1);
+    }
     if (prod < 1) prod = 1;
     const uint64_t frames = ((1ull << 24) - 1) / prod;
     const uint64_t kb = frames / 64;

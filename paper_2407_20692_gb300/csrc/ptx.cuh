@@ -25,6 +25,14 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 // another kernel reads or writes.  dep_launch() lets the next kernel's CTAs be
 // placed as soon as every CTA of this one has started (they wait in dep_wait()).
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A pointer to what the kernel before wrote, for use after dep_wait(): loads through
+// it depend on this point, so none (a read-only load least of all, which a compiler
+// may place anywhere) can be moved before the wait.
+template <typename T>
+__device__ __forceinline__ T* after_wait(T* p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------- packed FP32

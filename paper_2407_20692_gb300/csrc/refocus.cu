@@ -190,6 +190,8 @@ __global__ void __launch_bounds__(kBandThreads, 1) refocus_band_kernel(const __g
     }
     dep_wait();
     dep_launch();
+    const long long* const xcol = after_wait(g.xcol);
+    const long long* const xang = after_wait(g.xang);
     __syncthreads();
     if (tid == 0)
         for (uint32_t q = 0; q < (uint32_t)stages && q < total_sl; ++q) issue(q);
@@ -211,8 +213,8 @@ __global__ void __launch_bounds__(kBandThreads, 1) refocus_band_kernel(const __g
 #pragma unroll
         for (int j = 0; j < PT; ++j) {
             const int pj = p0 + min(j, np - 1);
-            X[j] = __ldg(g.xcol + (size_t)pj * kBandThreads + c) + __ldg(g.xang + 2 * pj);
-            dB[j] = __ldg(g.xang + 2 * pj + 1);
+            X[j] = __ldg(xcol + (size_t)pj * kBandThreads + c) + __ldg(xang + 2 * pj);
+            dB[j] = __ldg(xang + 2 * pj + 1);
         }
         // sums of plane pairs (2q, 2q + 1) in the two lanes of a packed register
         f32x2 U[PT / 2][KR], C[PT / 2][KR];
@@ -436,7 +438,9 @@ __global__ void __launch_bounds__(kBandThreads, 1) refocus_rows_kernel(const flo
     }
     dep_wait();
     dep_launch();
-    for (int p = tid; p < g.n_planes + PT; p += blockDim.x) step[p] = p < g.n_planes ? __ldg(g.xang + 2 * p + 1) : 0ll;
+    const long long* const xcol = after_wait(g.xcol);
+    const long long* const xang = after_wait(g.xang);
+    for (int p = tid; p < g.n_planes + PT; p += blockDim.x) step[p] = p < g.n_planes ? __ldg(xang + 2 * p + 1) : 0ll;
     __syncthreads();
     if (tid == 0)
         for (int q = 0; q < stages && (uint32_t)q < total_sl; ++q) issue(0, q, q);
@@ -458,7 +462,7 @@ __global__ void __launch_bounds__(kBandThreads, 1) refocus_rows_kernel(const flo
 #pragma unroll
         for (int j = 0; j < PT; ++j) {
             const int pj = p0 + min(j, np - 1);
-            X[j] = __ldg(g.xcol + (size_t)pj * kBandThreads + c) + __ldg(g.xang + 2 * pj);
+            X[j] = __ldg(xcol + (size_t)pj * kBandThreads + c) + __ldg(xang + 2 * pj);
         }
         // sums of row pairs (2h, 2h + 1) in the two lanes of a packed register
         f32x2 U[PT][KR / 2], C[PT][KR / 2];
@@ -614,7 +618,7 @@ __global__ void __launch_bounds__(kYThreads) refocus_ystage_kernel(const float* 
     dep_wait();      // the taps depend on nothing: formed while the x stage ends
     __syncthreads();
     const int64_t Ma = (int64_t)ha * wa;
-    const float* src = ubuf + (int64_t)p * hb * Ma;
+    const float* src = after_wait(ubuf) + (int64_t)p * hb * Ma;
     if ((wa & 3) == 0) {   // four adjacent columns per thread, 16-byte loads
         const int wq = wa >> 2;
         for (int idx = threadIdx.x; idx < RB * wq; idx += kYThreads) {

@@ -167,6 +167,7 @@ __global__ void __launch_bounds__(kColThreads, 1) r4_cols_kernel(const float* __
     }
     dep_launch();
     dep_wait();   // Gamma was complete before the tables' kernel began
+    t = after_wait(t);
     for (int p0 = 0; p0 < np; p0 += G) {
         const int gp = min(G, np - p0);
         __syncthreads();   // boxes ready / previous pass's tables consumed
@@ -242,6 +243,7 @@ __global__ void __launch_bounds__(kColThreadsG) r4_cols_global_kernel(const floa
     const float* gbase = g + ((int64_t)yb * wb) * ma + (int64_t)ya * wa;
     dep_wait();
     dep_launch();
+    t = after_wait(t);
     for (int p0 = 0; p0 < np; p0 += G) {
         const int gp = min(G, np - p0);
         __syncthreads();
@@ -307,6 +309,9 @@ __global__ void __launch_bounds__(kR4Threads) r4_rows_kernel(const float* __rest
     const int p = blockIdx.y;
     dep_wait();
     dep_launch();
+    t = after_wait(t);
+    c_hi = after_wait(c_hi);
+    c_lo = after_wait(c_lo);
     for (int w = threadIdx.x; w < G * wa; w += kR4Threads) {
         const int k = w / wa, xc = w - k * wa, xr = blockIdx.x * G + k;
         if (xr >= ha) continue;
