@@ -48,7 +48,7 @@ typedef enum cpi_status {
     CPI_OK = 0,
     CPI_ERR_INVALID_ARG = 1, /* a NULL/misaligned pointer, a bad size or descriptor */
     CPI_ERR_OVERFLOW = 2,    /* N^2 * max(A) * max(B) >= 2^63: int64 exactness not guaranteed */
-    CPI_ERR_WORKSPACE = 3,   /* workspace NULL or smaller than the size query */
+    CPI_ERR_WORKSPACE = 3,   /* workspace NULL, misaligned or too small (the size query's answer suffices) */
     CPI_ERR_UNSUPPORTED = 4, /* a valid request this build does not implement */
     CPI_ERR_CUDA = 5,        /* a CUDA runtime call or kernel launch failed */
     CPI_ERR_TIMEOUT = 6      /* a device-side wait ran out of its time limit */
@@ -111,8 +111,9 @@ CPI_API int32_t cpi_abi_version(void);
  * CPI_ERR_OVERFLOW); M_a, M_b <= 2^24; output pointers 16-byte aligned.
  * -------------------------------------------------------------------------- */
 
-/* Workspace bytes cpi_correlate / cpi_correlate_accumulate / cpi_correlate_stage
- * need for these descriptors and n_frames (0 on invalid arguments). */
+/* Workspace bytes that suffice for cpi_correlate / cpi_correlate_accumulate /
+ * cpi_correlate_stage with these descriptors and n_frames frames or fewer, such as
+ * an acquisition's last block (0 on invalid arguments). */
 CPI_API size_t cpi_correlate_workspace_size(const cpi_frames *a, const cpi_frames *b, int64_t n_frames);
 
 /* Whole Eq. (1): overwrites s_ab, s_a, s_b, and gamma / gamma_f32 when non-NULL. */
@@ -329,8 +330,9 @@ CPI_API cpi_status cpi_batch_correlate(const cpi_batch_item *items, int32_t n_it
  * CPI_NOALLOC_SCRATCH_BYTES that the library keeps in the device memory of every
  * GPU that loads it, until the process exits.  The call allocates nothing and
  * calls no allocating routine.
- *   - Problems whose workspace (cpi_correlate_workspace_size) exceeds
- *     CPI_NOALLOC_SCRATCH_BYTES are refused with CPI_ERR_WORKSPACE.
+ *   - Problems that need more scratch than CPI_NOALLOC_SCRATCH_BYTES (never those
+ *     whose cpi_correlate_workspace_size is within it) are refused with
+ *     CPI_ERR_WORKSPACE.
  *   - The first call on a device looks up the array's device address (set-up,
  *     once per device, with that device current); make that first call before
  *     any stream capture.

@@ -163,6 +163,7 @@ struct CorrPlan {
     int k_blocks, kb_per_chunk, n_chunks;
     int block_n, tiles_m, tiles_n, n_units;
     size_t off_a, off_b, off_part, off_vmax, off_sa, off_sb, ws_bytes;   // off_sa/off_sb: S_a, S_b when the caller passes none
+    size_t ws_upto;            // bytes that fit the plan of any frame count up to n, too
 };
 
 // split == 0: single correlation (more frame chunks when the tiles alone cannot
@@ -207,6 +208,7 @@ cpi_status make_plan_tiles(const cpi_frames* a, const cpi_frames* b, int64_t n, 
         if (want > max_by_len) want = max_by_len;
         if (want > n_chunks) n_chunks = want;
     }
+    const int asked_chunks = n_chunks;
     p.kb_per_chunk = (p.k_blocks + n_chunks - 1) / n_chunks;
     if (p.kb_per_chunk > max_kb_chunk) p.kb_per_chunk = max_kb_chunk;
     p.n_chunks = (p.k_blocks + p.kb_per_chunk - 1) / p.kb_per_chunk;
@@ -216,10 +218,16 @@ cpi_status make_plan_tiles(const cpi_frames* a, const cpi_frames* b, int64_t n, 
     p.off_a = 0;
     p.off_b = round_up(p.off_a + (size_t)p.Ma * (size_t)p.kstride_bytes, 1024);
     p.off_part = round_up(p.off_b + (size_t)p.Mb * (size_t)p.kstride_bytes, 1024);
-    p.off_vmax = round_up(p.off_part + (size_t)p.n_chunks * (size_t)p.Ma * (size_t)p.Mb * 4, 256);
-    p.off_sa = round_up(p.off_vmax + 2 * sizeof(uint32_t), 256);
-    p.off_sb = round_up(p.off_sa + (size_t)p.Ma * 8, 256);
-    p.ws_bytes = round_up(p.off_sb + (size_t)p.Mb * 8, 1024);
+    auto rest = [&](int slots) {   // what lies behind the operands
+        p.off_vmax = round_up(p.off_part + (size_t)slots * (size_t)p.Ma * (size_t)p.Mb * 4, 256);
+        p.off_sa = round_up(p.off_vmax + 2 * sizeof(uint32_t), 256);
+        p.off_sb = round_up(p.off_sa + (size_t)p.Ma * 8, 256);
+        return round_up(p.off_sb + (size_t)p.Mb * 8, 1024);
+    };
+    // The chunks asked for never fall as n grows; the whole K blocks per chunk can make
+    // fewer of them (9216 frames: 9 chunks of 4 K blocks, 10240: 8 of 5 instead of 10).
+    p.ws_upto = rest(asked_chunks);
+    p.ws_bytes = rest(p.n_chunks);
     *pl = p;
     return CPI_OK;
 }
@@ -236,7 +244,8 @@ double moments_cost(const CorrPlan& p, int sm_count) {
 
 // The plan of a single correlation: the tile width with the shorter raw-moment
 // launch (83x83 vs 37x37, N = 17321: 324 tiles of 256 columns in 3 waves, 594 of 128
-// in 4; 320 -> 275 us).  Narrow tiles never need more partial slots.
+// in 4; 320 -> 275 us).  Narrow tiles never ask for more partial slots, so the wide
+// plan's ws_upto holds for both.
 cpi_status make_plan(const cpi_frames* a, const cpi_frames* b, int64_t n, int sm_count, CorrPlan* pl) {
     CorrPlan wide, narrow;
     cpi_status s = make_plan_tiles(a, b, n, sm_count, &wide, 0, 256);
@@ -244,8 +253,10 @@ cpi_status make_plan(const cpi_frames* a, const cpi_frames* b, int64_t n, int sm
     *pl = wide;
     s = make_plan_tiles(a, b, n, sm_count, &narrow, 0, 128);
     if (s == CPI_OK && narrow.ws_bytes <= wide.ws_bytes &&
-        moments_cost(narrow, sm_count) < 0.95 * moments_cost(wide, sm_count))
+        moments_cost(narrow, sm_count) < 0.95 * moments_cost(wide, sm_count)) {
         *pl = narrow;
+        pl->ws_upto = wide.ws_upto;
+    }
     return CPI_OK;
 }
 
@@ -799,7 +810,7 @@ size_t cpi_correlate_workspace_size(const cpi_frames* a, const cpi_frames* b, in
     if (device_info(&dev) == cudaSuccess) sm = dev->sm_count;
     CorrPlan pl;
     if (make_plan(a, b, n_frames, sm, &pl) != CPI_OK) return 0;
-    return pl.ws_bytes;
+    return pl.ws_upto;
 }
 
 cpi_status cpi_correlate(const cpi_frames* a, const cpi_frames* b, int64_t n_frames,
