@@ -316,10 +316,10 @@ __global__ void __launch_bounds__(kConvThreads, 1) dnf_conv_kernel(const DnFlat 
         tmem_relinquish();
     }
     dep_wait();
-    dep_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    dep_launch();      // after the allocation is held (ptx.cuh)
     const uint32_t tmem_base = *tmem_slot;
 
     float bsum[MODE == kGrad ? 32 : 1];                         // epilogue: sums over this thread's pixels
@@ -896,10 +896,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
         tmem_relinquish();
     }
     dep_wait();
-    dep_launch();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    dep_launch();      // after the allocation is held (ptx.cuh)
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 4 && lane == 0) {

@@ -199,12 +199,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_relinquish();
     }
     dep_wait();
-    dep_launch();
     if constexpr (kBf16)
         for (int p = threadIdx.x; p < L.n_problems; p += blockDim.x) seg_kb[p] = segment_kblocks(L.prob[p]);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    dep_launch();      // after the allocation is held (ptx.cuh)
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t sf = tmem_base + (uint32_t)(C::kAcc * C::kBlockN);   // E2M1: block scales
     if constexpr (!kBf16) {

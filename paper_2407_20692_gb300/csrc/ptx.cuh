@@ -23,7 +23,12 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 // the stream is finishing: dep_wait() returns once that kernel is complete and its
 // writes are visible.  Every thread calls it before its first access to memory that
 // another kernel reads or writes.  dep_launch() lets the next kernel's CTAs be
-// placed as soon as every CTA of this one has started (they wait in dep_wait()).
+// placed as soon as every CTA of this one has started (they wait in dep_wait()).  A
+// kernel that allocates tensor memory calls it after the barrier that publishes its
+// allocation: a dependent CTA placed while the allocation still waits (for a kernel of
+// another stream on that SM) could allocate first and then wait for this kernel with
+// the columns it needs.  With that order whoever waits in dep_wait() holding columns
+// waits for CTAs that all hold theirs.
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // A pointer to what the kernel before wrote, for use after dep_wait(): loads through
 // it depend on this point, so none (a read-only load least of all, which a compiler
