@@ -18,6 +18,7 @@
 // to a whole number of CTA tiles.  The same pass adds the marginal sums
 // S_a = sum_i A_i (Eq. (1), second term) with exact int64 atomics.
 
+#include "frame_words.cuh"
 #include "kernels.cuh"
 #include "ptx.cuh"
 
@@ -273,7 +274,8 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t w, int lane) {
 }
 
 // Binary frames with 4-byte aligned frames.  CTA = (region, chunk of kWC frame words) x block of
-// kFB frames.  Words w0 .. w0 + kWC of every frame of the block are loaded with
+// kFB frames.  Words w0 .. w0 + kWC of every frame of the block, up to the region's
+// last byte (the caller's buffer may end there), are loaded with
 // coalesced 4-byte loads into shared memory, in rows of kWP words (kWP odd: a
 // warp reading one word of 32 frames touches 32 banks).  Each warp then takes
 // 32-pixel tiles of the region's rows (the last of a row may hold fewer pixels,
@@ -291,16 +293,6 @@ constexpr int kStageRow = kFB / 2 + 16;  // staged operand row (E2M1, two frames
 constexpr size_t kBitsSmem = sizeof(uint32_t) * kFB * kWP + (size_t)8 * 32 * kStageRow;
 static_assert(kWP % 2 == 1, "odd pitch");
 
-__host__ __device__ inline int64_t floor_div(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
-
-// First and last frame word a region's pixels occupy.
-__host__ __device__ inline int64_t region_first_word(const FramesDev& d) {
-    return ((int64_t)d.y0 * d.row_stride + d.x0) >> 5;
-}
-__host__ __device__ inline int64_t region_last_word(const FramesDev& d) {
-    return ((int64_t)(d.y0 + d.height - 1) * d.row_stride + d.x0 + d.width - 1) >> 5;
-}
-
 __global__ void __launch_bounds__(256) ingest_bits_kernel(FramesDev A, FramesDev B, int64_t n_frames, int64_t f_base,
                                                           int64_t kstride_bytes, uint8_t* op_a, uint8_t* op_b,
                                                           int64_t* s_a, int64_t* s_b, int chunks_a) {
@@ -317,21 +309,26 @@ __global__ void __launch_bounds__(256) ingest_bits_kernel(FramesDev A, FramesDev
     uint8_t* st = smem_bits + sizeof(uint32_t) * kFB * kWP + (size_t)warp * 32 * kStageRow;
 
     const int64_t w0 = region_first_word(d) + (int64_t)chunk * kWC;
-    const int64_t words_per_frame = d.frame_stride >> 2;
     const int64_t f0 = f_base + (int64_t)blockIdx.y * kFB;
     // asynchronous 4-byte copies (all of a thread's loads in flight at once);
-    // words past the frames or past a frame's end are zero-filled
+    // what lies past the frames or behind the region's last pixel is zero-filled
     // (warp w copies frames w, w + 8, ...; lane l words l and l + 32, lane 0 also word 64)
     static_assert(kWC == 64, "two words per lane plus one");
+    const int64_t whole = region_whole_words(d) - w0;       // words of the chunk up to the region's last byte
+    const int rest = region_rest_bytes(d);
+    auto within = [](int64_t n) { return (int)(n < 0 ? 0 : (n < kWC + 1 ? n : kWC + 1)); };
+    const int frames = (int)min((int64_t)kFB, n_frames - f0);
+    const int limit = within(whole + (rest != 0 ? 1 : 0)), limit_last = within(whole);
+    const int last = n_frames - f0 <= kFB ? frames - 1 : -1;   // its partial word is read below, byte by byte
     for (int fr = warp; fr < kFB; fr += 8) {
-        const int64_t f = f0 + fr;
-        const uint32_t* fbase = reinterpret_cast<const uint32_t*>(d.data + (f < n_frames ? f : 0) * d.frame_stride) + w0;
+        const int words = fr < frames ? (fr == last ? limit_last : limit) : 0;
+        const uint32_t* fbase = reinterpret_cast<const uint32_t*>(d.data + (f0 + fr) * d.frame_stride) + w0;
         const uint32_t sbase = static_cast<uint32_t>(__cvta_generic_to_shared(S + fr * kWP));
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const int w = k < 2 ? lane + 32 * k : 64;
+            const int w = k < 2 ? lane + 32 * k : kWC;
             if (k == 2 && lane != 0) break;
-            const bool in = f < n_frames && w0 + w < words_per_frame;
+            const bool in = w < words;
             const uint32_t* src = in ? fbase + w : reinterpret_cast<const uint32_t*>(d.data);
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(sbase + 4u * (uint32_t)w), "l"(src),
                          "r"(in ? 4 : 0)
@@ -340,6 +337,16 @@ __global__ void __launch_bounds__(256) ingest_bits_kernel(FramesDev A, FramesDev
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+    if (last >= 0 && limit > limit_last) {
+        if (threadIdx.x == 0) {
+            const uint8_t* p = d.data + (f0 + last) * d.frame_stride + 4 * (w0 + whole);
+            uint32_t v = p[0];
+            if (rest > 1) v |= (uint32_t)p[1] << 8;
+            if (rest > 2) v |= (uint32_t)p[2] << 16;
+            S[last * kWP + limit_last] = v;
+        }
+        __syncthreads();
+    }
 
     // rows with a tile whose first bit e0 = (y0 + y) rs + x0 + 32 xt lies in the chunk
     const int ntx = (d.width + 31) >> 5;
