@@ -4,9 +4,10 @@
 // packed one bit per pixel (Section 2 of the paper) or one byte per pixel.  The
 // raw-moment contraction sums over frames, so each operand row must hold one
 // pixel's values over consecutive frames (K-major):
-//   - 1-bit frames that start on 4-byte words -> FP4 E2M1 values packed two per byte (0x0 / 0x2 = 1.0; frame 2j in the low
-//     nibble of byte j), ingest_bits_kernel: a block of frames staged word-wise
-//     in shared memory, transposed 32 x 32 bits per warp;
+//   - 1-bit frames that start on 4-byte words, rows at least 8 pixels wide and not far
+//     apart (words_pay) -> FP4 E2M1 values packed two per byte (0x0 / 0x2 = 1.0; frame
+//     2j in the low nibble of byte j), ingest_bits_kernel: a block of frames staged
+//     word-wise in shared memory, transposed 32 x 32 bits per warp;
 //   - 8-bit frames with 4-pixel aligned regions -> BF16 (integers 0..255 are
 //     exact), ingest_u8x4_kernel: one CTA per tile of 128 pixels x 128 frames;
 //   - any other frames -> BF16 (1-bit frames that do not meet the first case as
@@ -401,7 +402,9 @@ __global__ void __launch_bounds__(256) ingest_bits_kernel(FramesDev A, FramesDev
 
 }  // namespace
 
-// Conditions of the word-load path for binary frames.
+// Conditions of the word-load path for binary frames.  A tile of 32 pixels costs the
+// same however few of its pixels a row fills: at 8 the paths are about equal (16x8 in
+// rows of 64: 12.5 us against 12.6; 64x8: 23 / 26), so narrower rows go bit by bit.
 static bool bits_fast_ok(const FramesDev& d) {
     return d.bits == 1 && d.width >= 8 && d.frame_stride % 4 == 0 &&
            reinterpret_cast<uintptr_t>(d.data) % 4 == 0;
@@ -425,7 +428,7 @@ cudaError_t launch_ingest(bool bf16, const FramesDev& a, const FramesDev& b, int
     }
     const int tiles_a = (int)((Ma + kIngestPixels - 1) / kIngestPixels);
     const int tiles_b = (int)((Mb + kIngestPixels - 1) / kIngestPixels);
-    if (!bf16 && bits_fast_ok(a) && bits_fast_ok(b) && (2 * kstride_bytes) % kFB == 0) {
+    if (!bf16 && bits_fast_ok(a) && bits_fast_ok(b) && words_pay(a, b) && (2 * kstride_bytes) % kFB == 0) {
         static bool attr[64] = {};
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);

@@ -33,12 +33,17 @@ int main() {
                 if (w < w0 || w > w1) return std::printf("pixel not covered\n"), 1;
             }
     }
+    // rows far apart: the words between them would be read for nothing
+    const Frames narrow{64, 8, 0, 0, 128}, apart{64, 8, 0, 0, 512}, wide{64, 31, 0, 0, 512}, lone{16, 50, 0, 0, 8192};
+    if (!cpi::words_pay(narrow, narrow) || cpi::words_pay(apart, apart) || !cpi::words_pay(wide, wide) ||
+        cpi::words_pay(lone, lone) || !cpi::words_pay(wide, apart))
+        return std::printf("words_pay\n"), 1;
     return 0;
 }
 """
 
 
-def test_words_cover_the_region_and_end_with_it(tmp_path):
+def test_words_cover_the_region_end_with_it_and_pay(tmp_path):
     src, exe = tmp_path / "words.cpp", tmp_path / "words"
     src.write_text(PROGRAM)
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(exe)], check=True)
