@@ -371,7 +371,7 @@ CPI_API cpi_status cpi_correlate_noalloc(const cpi_frames *a, const cpi_frames *
  * Requires ha, wa, hb, wb >= 1 and hb * wb <= 65535; errors are reported before
  * any launch.
  *
- * cpi_denoise      : gamma_out = denoised gamma_in (same layout).
+ * cpi_denoise      : gamma_out = denoised gamma_in (same layout; the two may overlap).
  * cpi_denoise_grad : training loss L = mean over all outputs of
  *                    (y - s * gamma_target)^2 into *loss (DEVICE float) and
  *                    dL/d(model) into grad (DEVICE float [CPI_DENOISER_PARAMS]).

@@ -260,7 +260,7 @@ struct ConvArgs {
     const float* bias;
     uint8_t* out;                 // kHidden: planes; kGrad: hi planes, which hold the activation; kTrain: records
     uint8_t* out_lo;              // kGrad
-    const float* gamma;           // last layer: the network's input
+    const float* gamma;           // last layer: the network's input (y_out may be the same buffer)
     const float* target;          // kTrain
     const float* scale;
     float* y_out;                 // kInfer
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) dnf_conv_kernel(const DnFlat 
                     float dy = 0.0f;
                     if (p.valid) {
                         const int64_t o = (int64_t)p.b * HW + (int64_t)p.y * g.W + p.x;
-                        const float xcen = bf16r(__ldg(a.gamma + o) * sc);
+                        const float xcen = bf16r(a.gamma[o] * sc);
                         const float y = xcen + (__uint_as_float(r[0]) + __ldg(a.bias));
                         if constexpr (MODE == kInfer) {
                             a.y_out[o] = y / sc;
@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(kExThreads, 2) dnf_conv_exact_kernel(const DnF
                 float dy = 0.0f;
                 if (px.valid) {
                     const int64_t o = (int64_t)px.b * HW + (int64_t)px.y * g.W + px.x;
-                    const float y = bf16r(__ldg(a.gamma + o) * sc) + (acc1[p] + __ldg(a.bias));
+                    const float y = bf16r(a.gamma[o] * sc) + (acc1[p] + __ldg(a.bias));
                     if constexpr (MODE == kInfer) {
                         a.y_out[o] = y / sc;
                     } else {
@@ -1244,8 +1244,15 @@ bool dn_flat_plan(int ha, int wa, int hb, int wb, bool training, size_t ws_bytes
 cudaError_t dn_flat_denoise(const DnFlat& g, const float* model, const float* gamma_in, float* gamma_out, int hb, int wb,
                             uint8_t* ws, int sm_count, unsigned int* status, unsigned long long timeout_ns,
                             cudaStream_t st) {
+    const int64_t n = (int64_t)hb * wb * g.H * g.W;
     uint8_t* x = ws + g.act[0];
     uint8_t* c = ws + g.act[1];
+    // The last layer reads the input pixel by pixel as it writes the output, and FP32
+    // layers read the model: an output that overlaps them otherwise than in place goes
+    // through the workspace.
+    auto on = [&](const float* p, int64_t len) { return gamma_out < p + len && p < gamma_out + n; };
+    const bool apart = (gamma_out == gamma_in || !on(gamma_in, n)) && !on(model, kDenoiserParams);
+    float* y = apart ? gamma_out : reinterpret_cast<float*>(x);
     const uint8_t* wt = ws + g.wt;
     const Margins mg{{x, c}, 2};
     cudaError_t e = launch_inputs(g, gamma_in, model, hb, wb, ws, x, mg, kWFwdElems, sm_count, st);
@@ -1259,8 +1266,10 @@ cudaError_t dn_flat_denoise(const DnFlat& g, const float* model, const float* ga
     a.in = x, a.out = c, a.wt += 2 * kW1Elems, a.bias = model + kPB2;
     if (e == cudaSuccess) e = launch_forward<32, 32, kHidden>(g, a, model + kPW2, sm_count, st);
     a.in = c, a.out = nullptr, a.wt += 2 * kW1Elems, a.bias = model + kPB3;
-    a.gamma = gamma_in, a.scale = reinterpret_cast<const float*>(ws + g.scale), a.y_out = gamma_out;
+    a.gamma = gamma_in, a.scale = reinterpret_cast<const float*>(ws + g.scale), a.y_out = y;
     if (e == cudaSuccess) e = launch_forward<32, 1, kInfer>(g, a, model + kPW3, sm_count, st);
+    if (e == cudaSuccess && !apart)
+        e = cudaMemcpyAsync(gamma_out, y, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, st);
     return e;
 }
 
