@@ -362,7 +362,10 @@ CPI_API cpi_status cpi_correlate_noalloc(const cpi_frames *a, const cpi_frames *
  *   a1 = relu(conv(x; 9 -> 32)), a2 = relu(conv(a1; 32 -> 32)),
  *   a3 = relu(conv(a2; 32 -> 32)), y = x[4] + conv(a3; 32 -> 1)
  *   (3 x 3 kernels, zero padding 1, with biases); gamma_out = y / s.
- * x, a1..a3 and the weights in use are rounded to bfloat16; sums are float32.
+ * x, a1..a3 and the weights in use are rounded to bfloat16; sums are float32 (those
+ * on the tensor cores truncated after each step: the forward layers at widths 32, 64
+ * and 128, and the gradients, whose terms at the hidden layers are held as two
+ * bfloat16 values each).
  *
  * model: DEVICE float [CPI_DENOISER_PARAMS], float32 master weights, per layer
  *   l = 0..3 the weights W_l [Cout][Cin][3][3] then the biases b_l [Cout].

@@ -808,8 +808,11 @@ __global__ void __launch_bounds__(kTopThreads) dnf_top_grad_kernel(const DnFlat 
 // lane of it) issues, warps 0..3 add every unit's sums to FP32 registers while the next
 // unit runs into the other accumulator: tensor-core sums are truncated, so an
 // accumulator left to grow over all of a CTA's pixels is biased in proportion to
-// their number (measured on the last layer, whose terms cancel: 7.4e-6 of the
-// gradient at 80x80 vs 12x12 against 4.6e-7 in FP32).  hold: images 64 wide, whose
+// their number (measured on the last layer: 7.4e-6 of the gradient at 80x80 vs 12x12
+// against 4.6e-7 in FP32).  The last layer's gradients, exact but for these sums, go in
+// runs of 64 pixels: over 28 training steps of widths 24 to 128 the error of the whole
+// gradient against 64 bits is 0.98 of that of FP32 sums (1.02 at most), with runs of a
+// unit it was 1.00 (1.07 at most, always above 1 at widths 32 and 128).  hold: images 64 wide, whose
 // gradients have always been summed that way, keep one accumulator to the end over
 // the same blocks of up to 32 rows of a slice per CTA, so that training there goes
 // on as it was.  1024 slices of 64 x 64, 32 -> 32: 194 us, 0.83 GB at 4.3 TB/s.  At the
@@ -857,7 +860,8 @@ struct WgWalk {
     }
 };
 
-template <int KC, int NB>
+// kRun: K steps (16 pixels) per run, 0: a unit's, or all of a CTA's (hold)
+template <int KC, int NB, int kRun>
 __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g, const WgArgs a) {
     constexpr int kDPlanes = NB / 8;                       // staged delta planes (NB = 16: the second stays unused)
     constexpr uint32_t kCols = 3 * NB;
@@ -950,16 +954,37 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
             tc_fence_after();
             const int steps = (int)min(w.left, (int64_t)a.U) / 16;
             const uint32_t base = smem_u32(ring + (size_t)s * stage_bytes);
-            const uint32_t d = tmem_base + (uint32_t)acc * kCols;
+            uint32_t d = tmem_base + (uint32_t)acc * kCols;
             uint64_t bd = sdesc_plain(base, 128, dplane);
             uint64_t ad = sdesc_plain(base + kDPlanes * dplane, 128, aplane);
-            for (int k = 0; k < steps; ++k, ad += 16, bd += 16) {
+            auto sum = [&](int n, bool fresh) {
+                for (int k = 0; k < n; ++k, ad += 16, bd += 16) {
 #pragma unroll
-                for (int ky = 0; ky < 3; ++ky)
-                    umma_bf16(on, d + (uint32_t)(ky * NB), ad + (uint64_t)(uint32_t)(ky * a.bstride), bd, idesc,
-                                   first && k == 0 ? 0u : 1u);
+                    for (int ky = 0; ky < 3; ++ky)
+                        umma_bf16(on, d + (uint32_t)(ky * NB), ad + (uint64_t)(uint32_t)(ky * a.bstride), bd, idesc,
+                                       fresh && k == 0 ? 0u : 1u);
+                }
+            };
+            if constexpr (kRun == 0) {
+                sum(steps, first);
+            } else {
+                sum(min(kRun, steps), true);
+                for (int k = kRun; k < steps; k += kRun) {      // the next run: the other accumulator
+                    umma_commit(on, &tfull[acc]);
+                    if (++acc == 2) {
+                        acc = 0;
+                        acc_phase ^= 1;
+                    }
+                    ok = __all_sync(0xffffffffu,
+                                    mbar_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, a.status, a.timeout_ns));
+                    if (!ok) break;
+                    tc_fence_after();
+                    d = tmem_base + (uint32_t)acc * kCols;
+                    sum(min(kRun, steps - k), true);
+                }
             }
             any = true;
+            if (!ok) break;
             umma_commit(on, &empty[s]);
             if (++s == stages) {
                 s = 0;
@@ -983,7 +1008,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
         bool ok = true;
         int acc = 0;
         uint32_t acc_phase = 0;
-        for (int v = blockIdx.x; v < a.n_blocks; v += a.hold ? a.n_blocks : (int)gridDim.x) {
+        int left = 0;                                       // K steps of the unit still to come
+        for (int v = blockIdx.x; v < a.n_blocks;) {
+            if (kRun > 0 && left == 0)
+                left = (int)min((int64_t)a.U, ((int64_t)g.Q + 15) / 16 * 16 - (int64_t)v * a.U) / 16;
             if (!mbar_wait_bounded(&tfull[acc], acc_phase, abort_flag, a.status, a.timeout_ns)) {
                 ok = false;
                 break;
@@ -1004,6 +1032,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
                 acc = 0;
                 acc_phase ^= 1;
             }
+            if (a.hold) break;
+            left = kRun > 0 ? max(0, left - kRun) : 0;
+            if (left == 0) v += (int)gridDim.x;
         }
         const int row = 32 * warp + lane;
         if (ok && row < kRows) {
@@ -1149,12 +1180,12 @@ cudaError_t launch_forward(DnFlat g, const ConvArgs& a, const float* w, int sm_c
     return launch_kernel(in_chain(g), dnf_conv_exact_kernel<CIN, COUT, MODE>, grid, kExThreads, smem, st, g, a, w);
 }
 
-template <int CIN, int KC, int COUT>
+template <int CIN, int KC, int COUT, int kRun = 0>
 cudaError_t launch_wgrad(const DnFlat& g, WgArgs a, const float* bias_part, int nbias, const double* loss_part, int nloss,
                          int64_t n, float* grad, float* loss, int sm_count, cudaStream_t st) {
     constexpr int NB = COUT == 32 ? 64 : 16;
     static bool attr[64] = {};
-    cudaError_t e = allow_smem(dnf_wgrad_kernel<KC, NB>, attr);
+    cudaError_t e = allow_smem(dnf_wgrad_kernel<KC, NB, kRun>, attr);
     if (e != cudaSuccess) return e;
     // pixels per unit: up to 256 (the staged halo of two rows is shared by more of
     // them), fewer when two stages do not fit or SMs would stay idle
@@ -1180,7 +1211,7 @@ cudaError_t launch_wgrad(const DnFlat& g, WgArgs a, const float* bias_part, int 
     if (a.stages > kWgMaxStages) a.stages = kWgMaxStages;
     int grid = a.n_blocks < sm_count ? a.n_blocks : sm_count;
     if (grid > kDnMaxCtas) grid = kDnMaxCtas;
-    e = launch_kernel(in_chain(g), dnf_wgrad_kernel<KC, NB>, grid, kWgThreads, 256 + a.stages * stage + a.slack, st, g, a);
+    e = launch_kernel(in_chain(g), dnf_wgrad_kernel<KC, NB, kRun>, grid, kWgThreads, 256 + a.stages * stage + a.slack, st, g, a);
     if (e != cudaSuccess) return e;
     return launch_kernel(in_chain(g), dnf_wgrad_reduce_kernel<CIN, KC, COUT>, 9 * CIN + 1, 256, 0, st, a.part, grid,
         bias_part, nbias, loss_part, nloss, n, grad, loss);
@@ -1312,7 +1343,9 @@ cudaError_t dn_flat_grad(const DnFlat& g, const float* model, const float* gamma
     w.status = status;
     w.timeout_ns = timeout_ns;
     w.in = act[2], w.d_hi = rec;
-    if (e == cudaSuccess) e = launch_wgrad<32, 4, 1>(g, w, bpart[3], top, sums, top, n, grad + kPW3, loss, sm_count, st);
+    if (e == cudaSuccess)
+        e = w.hold ? launch_wgrad<32, 4, 1>(g, w, bpart[3], top, sums, top, n, grad + kPW3, loss, sm_count, st)
+                   : launch_wgrad<32, 4, 1, 4>(g, w, bpart[3], top, sums, top, n, grad + kPW3, loss, sm_count, st);
     if (e == cudaSuccess) {
         const int64_t blocks = ((int64_t)g.Q + kTopPixels - 1) / kTopPixels;
         nb[2] = (int)(blocks < kTopCtas ? blocks : kTopCtas);
