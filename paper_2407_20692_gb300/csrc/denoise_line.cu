@@ -822,7 +822,8 @@ __global__ void __launch_bounds__(kTopThreads) dnf_top_grad_kernel(const DnFlat 
 // unit it was 1.00 (1.07 at most, always above 1 at widths 32 and 128).  hold: images 64 wide, whose
 // gradients have always been summed that way, keep one accumulator to the end over
 // the same blocks of up to 32 rows of a slice per CTA, so that training there goes
-// on as it was.  1024 slices of 64 x 64, 32 -> 32: 194 us, 0.83 GB at 4.3 TB/s.  At the
+// on as it was; only the first unit has an accumulator of its own, which makes up for
+// the zero column that is summed with every row.  1024 slices of 64 x 64, 32 -> 32: 194 us, 0.83 GB at 4.3 TB/s.  At the
 // end the CTA writes rows (kx, ci) x
 // columns (ky, n) to part[cta].  Every wait is bounded.
 constexpr int kWgThreads = 192;
@@ -949,11 +950,11 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
         constexpr uint32_t idesc = idesc_bf16(128, NB) | (1u << 15) | (1u << 16);
         const uint32_t on = elect_one() ? 1u : 0u;
         bool ok = true, any = false;
-        int s = 0, acc = 0;
+        int s = 0, acc = 0, units = 0;
         uint32_t phase = 0, acc_phase = 0;
         WgWalk w;
-        for (w.block(g, a, (int)blockIdx.x); w.live(a); w.next(g, a)) {
-            const bool first = !a.hold || !any, last = !a.hold || w.last(a);
+        for (w.block(g, a, (int)blockIdx.x); w.live(a); w.next(g, a), ++units) {
+            const bool first = !a.hold || units < 2, last = !a.hold || units == 0 || w.last(a);
             ok = (!first || mbar_wait_bounded(&tempty[acc], acc_phase ^ 1, abort_flag, a.status, a.timeout_ns)) &&
                  mbar_wait_bounded(&full[s], phase, abort_flag, a.status, a.timeout_ns);
             ok = __all_sync(0xffffffffu, ok);
@@ -1016,6 +1017,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
         int acc = 0;
         uint32_t acc_phase = 0;
         int left = 0;                                       // K steps of the unit still to come
+        WgWalk w;
+        w.block(g, a, (int)blockIdx.x);
+        bool more = a.hold && !w.last(a);                   // hold: the sums of the units after the first
         for (int v = blockIdx.x; v < a.n_blocks;) {
             if (kRun > 0 && left == 0)
                 left = (int)min((int64_t)a.U, ((int64_t)g.Q + 15) / 16 * 16 - (int64_t)v * a.U) / 16;
@@ -1039,7 +1043,11 @@ __global__ void __launch_bounds__(kWgThreads, 1) dnf_wgrad_kernel(const DnFlat g
                 acc = 0;
                 acc_phase ^= 1;
             }
-            if (a.hold) break;
+            if (a.hold) {
+                if (!more) break;
+                more = false;
+                continue;
+            }
             left = kRun > 0 ? max(0, left - kRun) : 0;
             if (left == 0) v += (int)gridDim.x;
         }

@@ -23,8 +23,7 @@ def _ready(cuda_ready):
     yield
 
 
-@pytest.mark.parametrize("hb,wb,ha,wa", [(16, 16, 32, 32), (12, 11, 30, 128), (13, 16, 29, 41), (16, 16, 60, 33)])
-def test_sums_of_one_sign_are_not_biased(hb, wb, ha, wa):
+def _relative_errors(hb, wb, ha, wa):
     rng = np.random.default_rng(ha * 100 + wa)
     g = (0.01 * rng.standard_normal((hb * wb, ha * wa))).astype(np.float32)
     t = (-0.05 - 0.01 * rng.random(g.shape)).astype(np.float32)
@@ -51,4 +50,16 @@ def test_sums_of_one_sign_are_not_biased(hb, wb, ha, wa):
                 want[i, ky, kx] = (dy * p[:, ky:ky + ha, kx:kx + wa]).sum()
     want = want.repeat(16, 1, 1)
     got = grad[at[3]:at[3] + 288].view(32, 3, 3).cpu().double()
-    assert ((got - want) / want).abs().max().item() <= 2e-7
+    return (got - want) / want
+
+
+@pytest.mark.parametrize("hb,wb,ha,wa", [(16, 16, 32, 32), (12, 11, 30, 128), (13, 16, 29, 41), (16, 16, 60, 33)])
+def test_sums_of_one_sign_are_not_biased(hb, wb, ha, wa):
+    assert _relative_errors(hb, wb, ha, wa).abs().max().item() <= 2e-7
+
+
+def test_bias_at_64_wide_is_no_larger_than_that_of_the_images_own_pixels():
+    """Images 64 wide sum a CTA's pixels in tensor-core accumulators to the end: 8.09e-6
+    low at this size in one accumulator over the pixels of the images, 8.20e-6 with the
+    zero column of the padded line summed too."""
+    assert _relative_errors(12, 16, 60, 64).mean().abs().item() <= 8.1e-6
