@@ -25,7 +25,10 @@ namespace {
 
 constexpr int kMaxTiles = 4;                // 128-pixel tiles per unit
 constexpr int kLineRound = 1024;            // the longest unit of any pass (512 on the tensor cores)
-constexpr uint32_t kShortLine = 1u << 15;   // positions: below, units of one tile
+// Positions: below, units of one tile (which lines under 304 x 256 positions, two units
+// per SM, take for their speed anyway) and margins of 128, not 512 positions, so that
+// small images' lines fit the workspace.
+constexpr uint32_t kShortLine = 1u << 15;
 constexpr int kMaxStages = 4;
 constexpr int kConvThreads = 320;           // warp 0 copies, warp 1 issues MMAs, warps 2..9 epilogue
 constexpr int kEpiThreads = 256;
@@ -1121,9 +1124,15 @@ __global__ void __launch_bounds__(256) dnf_wgrad_reduce_kernel(const float* __re
 }
 
 // ------------------------------------------------------------------ host
-// Short lines gain from kernels placed ahead (42x64 vs 12x9: 86 -> 77 us a call); on
-// long ones the gaps do not count and it costs (64x64 vs 32x32: 514 -> 546 us).
-bool in_chain(const DnFlat& g) { return g.Q < (1u << 20); }
+// Short lines at the tensor-core widths gain from kernels placed ahead, on long ones the
+// gaps do not count and the placed CTAs cost.  Chained and plain, us: 32x64 vs 8x9 (154
+// thousand positions) 56 / 62, 64x64 vs 14x16 (946 thousand) 169 / 171, 32x32 vs 31x32
+// (1.08 million) 180 / 182, 64x64 vs 20x20 (1.69 million) 253 / 248, 64x64 vs 32x32 547 /
+// 517; training 182 / 209, 569 / 587, 632 / 651, 922 / 936, 2052 / 2029.  The FP32
+// kernels fill an SM's registers, so whatever is placed ahead takes a CTA's place: 24x31
+// vs 8x8 136 / 117, 47x53 vs 10x12 421 / 377, 83x83 vs 20x20 2591 / 2482 (training 3858 /
+// 3706).
+bool in_chain(const DnFlat& g) { return g.tensor && g.Q < (1u << 20); }
 
 template <typename K>
 cudaError_t allow_smem(K kernel, bool (&done)[64]) {
