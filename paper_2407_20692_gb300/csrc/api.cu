@@ -232,20 +232,26 @@ cpi_status make_plan_tiles(const cpi_frames* a, const cpi_frames* b, int64_t n, 
     return CPI_OK;
 }
 
-// Length of the raw-moment launch: its waves of units times a unit's time, in cycles
-// of a 128 x 256 tile's K block (512) and of its epilogue.  A tile of half the width
-// takes 0.62 of the time (measured: 128x128 vs 64x64, N = 50000, 27 waves in 4.32 ms
-// against 14 in 3.64 ms; it reads as much of A from shared memory for half the
-// columns), so it pays where it fills the last wave or the last column tile better.
+// Length of the raw-moment launch in us: its waves of units times a unit's K blocks and
+// its epilogue, which costs several times as much where rows of the partial sums are not
+// whole 16-byte words.  After the launches of 95 shapes (24x16 to 128x128 against 8x8 to
+// 128x128 pixels, 1500 to 50000 frames) timed at both widths, which a straight line of
+// this form meets within 6% rms.
 double moments_cost(const CorrPlan& p, int sm_count) {
-    const double unit = (double)p.kb_per_chunk * 512.0 + 2500.0;
-    return (double)((p.n_units + sm_count - 1) / sm_count) * unit * (p.block_n == 128 ? 0.62 : 1.0);
+    static const double kBlock[2][2] = {{0.33, 0.205}, {0.340, 0.214}};                       // [bf16][narrow]
+    static const double kEpilogue[2][2][2] = {{{4.0, 2.0}, {19.5, 10.0}}, {{0.5, 0.3}, {14.7, 6.8}}};   // [bf16][ragged][narrow]
+    const int narrow = p.block_n == 128, ragged = p.Mb % 4 != 0;
+    const double unit = p.kb_per_chunk * kBlock[p.bf16][narrow] + kEpilogue[p.bf16][ragged][narrow];
+    return (double)((p.n_units + sm_count - 1) / sm_count) * unit;
 }
 
-// The plan of a single correlation: the tile width with the shorter raw-moment
-// launch (83x83 vs 37x37, N = 17321: 324 tiles of 256 columns in 3 waves, 594 of 128
-// in 4; 320 -> 275 us).  Narrow tiles never ask for more partial slots, so the wide
-// plan's ws_upto holds for both.
+// The plan of a single correlation: the tile width with the shorter raw-moment launch.
+// Wide and narrow, us: binary 64x64 vs 32x32, N = 20000: 31.9 / 43.7; 83x83 vs 37x37,
+// 17321: 122 / 95; 28x52 vs 39x29, 4772: 31 / 21; 128x128 vs 128x128, 32768: 2549 / 3128;
+// counts 83x83 vs 37x37, 17321: 324 / 277; 128x128 vs 64x64, 50000: 3949 / 4573.  Over
+// the 95 shapes the width taken costs 0.6% more than the better one on average, one
+// ratio of the widths for all of them (0.62) 3.6%, wide tiles everywhere 7%.  Narrow tiles
+// never ask for more partial slots, so the wide plan's ws_upto holds for both.
 cpi_status make_plan(const cpi_frames* a, const cpi_frames* b, int64_t n, int sm_count, CorrPlan* pl) {
     CorrPlan wide, narrow;
     cpi_status s = make_plan_tiles(a, b, n, sm_count, &wide, 0, 256);
@@ -253,7 +259,7 @@ cpi_status make_plan(const cpi_frames* a, const cpi_frames* b, int64_t n, int sm
     *pl = wide;
     s = make_plan_tiles(a, b, n, sm_count, &narrow, 0, 128);
     if (s == CPI_OK && narrow.ws_bytes <= wide.ws_bytes &&
-        moments_cost(narrow, sm_count) < 0.95 * moments_cost(wide, sm_count)) {
+        moments_cost(narrow, sm_count) < 0.97 * moments_cost(wide, sm_count)) {
         *pl = narrow;
         pl->ws_upto = wide.ws_upto;
     }
