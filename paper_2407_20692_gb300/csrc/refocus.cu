@@ -780,6 +780,13 @@ cudaError_t launch_band(const BandPlan& b, const CUtensorMap* tm, const BandGeom
     }
 }
 
+// Output rows per y-stage CTA: its y taps (rows x hb entries) fit in 200 KiB.
+int y_rows_per_cta(int hb) {
+    int rb = (int)((200 * 1024) / ((size_t)hb * sizeof(YTap)));
+    if (rb > 8) rb = 8;
+    return rb;
+}
+
 // The interleaved form: its row sets, rows and planes per thread, and how the call's
 // planes are split into launches.  The copy of Gamma shares the workspace with the
 // x-stage images, so it needs a call of enough planes: the images of a launch's
@@ -791,7 +798,7 @@ struct RowPlan {
     size_t stage_bytes, smem, copy_off;
 };
 
-RowPlan row_plan(int ha, int wa, int hb, int wb, int n_planes, size_t image_bytes, int sm_count) {
+RowPlan row_plan(const BandPlan& band, int ha, int wa, int hb, int wb, int n_planes, size_t image_bytes, int sm_count) {
     RowPlan b{};
     const size_t Ma = (size_t)ha * wa;
     b.groups = (ha + 3) / 4;
@@ -840,14 +847,34 @@ RowPlan row_plan(int ha, int wa, int hb, int wb, int n_planes, size_t image_byte
     // against 312).
     const int64_t units = (int64_t)hb * ((b.chunk + b.PT - 1) / b.PT) * b.n_bands;
     if (units * (b.threads / 32) < 2 * (int64_t)sm_count * 16) b.ok = false;
+    // Else the form with the shorter call.  x stage: 1970 samples a ns with every lane
+    // and unit in use, a tenth faster interleaved; its units come in whole waves, and the
+    // copy may split the planes over more launches and so more last waves.  Each launch
+    // added takes 4 us and a y stage, which takes as long for fewer planes where it does
+    // not fill the GPU: per angular row 0.12 us for 256 outputs of a CTA (0.15 for 1024
+    // where they are read as vectors).  Row-major and interleaved, us: 26x411 vs 40x2 with
+    // 24 planes 106 / 171; 57x60 vs 63x18, 42: 149 / 190; 119x126 vs 42x61, 23: 657 / 606;
+    // 61x90 vs 56x48, 64: 760 / 604; 96x96 vs 40x40, 128: 1336 / 1042.  Over 310 stacks timed
+    // in both forms (4 to 254 rows, 8 to 512 wide, 2 to 95 angular rows) the form taken costs
+    // 0.4% more than the better one on average, the interleaved one wherever it fits 4.2%;
+    // at 1.07 none of them is row-major where that is over 2% the slower one.
+    auto x_us = [&](int per_unit, int bands, int band_rows, int threads, int columns, int64_t slots, int chunk) {
+        double t = 0.0;
+        for (int p0 = 0; p0 < n_planes; p0 += chunk) {
+            const int np = n_planes - p0 < chunk ? n_planes - p0 : chunk;
+            const int64_t u = (int64_t)hb * ((np + per_unit - 1) / per_unit) * bands;
+            t += (double)((u + slots - 1) / slots * slots) / (double)u * np;
+        }
+        return t * bands * band_rows * wa * threads / columns * hb * wb / 1.97e6;
+    };
+    const int added = launches - (n_planes + kRefocusMaxPlanesPerLaunch - 1) / kRefocusMaxPlanesPerLaunch;
+    const int RB = y_rows_per_cta(hb);
+    const double y_idle = 1.0 - (double)((ha + RB - 1) / RB) * b.chunk / 400.0;
+    const double y_us = hb * (wa % 4 ? 0.12 * ((RB * wa + 255) / 256) : 0.15 * ((RB * wa / 4 + 255) / 256));
+    const double rows_us = 0.9 * x_us(b.PT, b.n_bands, b.R * b.KR, b.threads, b.R * wa, (int64_t)sm_count * b.per_sm, b.chunk) +
+                           added * (4.0 + (y_idle > 0.0 ? y_idle : 0.0) * y_us);
+    if (rows_us >= 1.07 * x_us(band.PB, band.n_bands, band.BH, band.cwt, wa, sm_count, kRefocusMaxPlanesPerLaunch)) b.ok = false;
     return b;
-}
-
-// Output rows per y-stage CTA: its y taps (rows x hb entries) fit in 200 KiB.
-int y_rows_per_cta(int hb) {
-    int rb = (int)((200 * 1024) / ((size_t)hb * sizeof(YTap)));
-    if (rb > 8) rb = 8;
-    return rb;
 }
 
 size_t round256(size_t x) { return (x + 255) / 256 * 256; }
@@ -892,7 +919,7 @@ cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, 
     long long* xcol = reinterpret_cast<long long*>(ws + tab_off);
     long long* xang = reinterpret_cast<long long*>(
         ws + tab_off + round256((size_t)kRefocusMaxPlanesPerLaunch * kBandThreads * sizeof(long long)));
-    const RowPlan rw = row_plan(ha, wa, hb, wb, n_planes, tab_off, sm_count);
+    const RowPlan rw = row_plan(b, ha, wa, hb, wb, n_planes, tab_off, sm_count);
     cudaError_t e = cudaSuccess;
     CUtensorMap tm;
     const float* gi = nullptr;

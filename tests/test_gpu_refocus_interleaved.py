@@ -43,9 +43,9 @@ def _run(g, copy, ha, wa, hb, wb, alpha, beta):
 
 
 @pytest.mark.parametrize("ha,wa,hb,wb,n", [
-    (83, 83, 37, 37, 128), (61, 32, 40, 25, 150), (130, 128, 12, 16, 48), (45, 100, 24, 11, 129), (9, 260, 60, 20, 61),
-    (18, 512, 40, 17, 40), (96, 96, 20, 31, 300), (13, 7, 200, 5, 300), (37, 250, 30, 9, 95), (70, 50, 30, 29, 127),
-    (3, 31, 400, 3, 102), (40, 40, 160, 1, 128)])
+    (83, 83, 37, 37, 128), (61, 32, 40, 25, 150), (130, 128, 12, 16, 128), (45, 100, 24, 11, 129), (9, 260, 20, 60, 119),
+    (202, 512, 10, 2, 61), (96, 96, 20, 31, 300), (13, 7, 200, 5, 300), (37, 250, 30, 9, 95), (70, 50, 30, 29, 127),
+    (3, 31, 400, 3, 103), (40, 40, 160, 1, 128)])
 def test_interleaved_form_equals_row_major(ha, wa, hb, wb, n):
     rng = np.random.default_rng(ha * 1000 + wa)
     g = torch.tensor(rng.standard_normal((hb * wb, ha * wa)).astype(np.float32), device="cuda")
@@ -58,3 +58,12 @@ def test_interleaved_form_equals_row_major(ha, wa, hb, wb, n):
         one, form = _run(g, copy, ha, wa, hb, wb, alpha[p:p + 1], beta[p:p + 1])
         assert not form
         assert torch.equal(full[p].view(torch.int32), one[0].view(torch.int32)), p
+
+
+@pytest.mark.parametrize("ha,wa,hb,wb,n", [(26, 411, 40, 2, 24), (13, 442, 43, 24, 34), (57, 60, 63, 18, 42)])
+def test_stacks_that_the_copy_splits_for_nothing(ha, wa, hb, wb, n):
+    """The copy would split these stacks, and their y stages do not fill the GPU or the
+    last waves of units weigh more."""
+    g = torch.zeros((hb * wb, ha * wa), dtype=torch.float32, device="cuda")
+    alpha = np.linspace(0.5, 1.5, n)
+    assert not _run(g + 1.0, _interleaved(g + 1.0, ha, wa), ha, wa, hb, wb, alpha, 1.0 - alpha)[1]
