@@ -140,9 +140,9 @@ __device__ __forceinline__ void r4_sample2(f32x2& acc, f32x2& cmp, f32x2 fa, f32
     r4_kahan2(acc, cmp, fma2(fb, bot, mul2(gb, top)));
 }
 
-constexpr int kColThreads = 1024;      // at most; 512 where two CTAs fit an SM
-template <int K>
-__global__ void __launch_bounds__(kColThreads, 1) r4_cols_kernel(const float* __restrict__ g, int np, int G, int ha,
+constexpr int kColThreads = 1024;      // at most; 512 where two or three CTAs fit an SM
+template <int K, int kCtas>
+__global__ void __launch_bounds__(kCtas == 3 ? 512 : kColThreads, kCtas == 3 ? 3 : 1) r4_cols_kernel(const float* __restrict__ g, int np, int G, int ha,
                                                                  int wa, int hb, int wb, int WP,
                                                                  const long long* __restrict__ t, int64_t stride,
                                                                  float* __restrict__ c_hi, float* __restrict__ c_lo) {
@@ -404,8 +404,8 @@ ColPlan r4_col_plan(int ha, int wa, int hb, int wb, int np, double skew) {
     return {};
 }
 
-template <int K>
-cudaError_t launch_cols(const ColPlan& c, const float* g, int np, int ha, int wa, int hb, int wb, const long long* t,
+template <int K, int kCtas>
+cudaError_t launch_cols_t(const ColPlan& c, const float* g, int np, int ha, int wa, int hb, int wb, const long long* t,
                         int64_t stride, float* c_hi, float* c_lo, cudaStream_t st) {
     static bool attr[64] = {};
     int dev = 0;
@@ -413,14 +413,29 @@ cudaError_t launch_cols(const ColPlan& c, const float* g, int np, int ha, int wa
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!attr[dev]) {
-        if ((e = cudaFuncSetAttribute(r4_cols_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kR4SmemCap)) !=
+        if ((e = cudaFuncSetAttribute(r4_cols_kernel<K, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kR4SmemCap)) !=
             cudaSuccess)
             return e;
         attr[dev] = true;
     }
     const dim3 grid((unsigned)hb, (unsigned)((ha + K - 1) / K));
-    return launch_kernel(true, r4_cols_kernel<K>, grid, c.threads, c.smem, st, g, np, c.G, ha, wa, hb, wb, c.WP, t, stride,
+    return launch_kernel(true, r4_cols_kernel<K, kCtas>, grid, c.threads, c.smem, st, g, np, c.G, ha, wa, hb, wb, c.WP, t, stride,
                          c_hi, c_lo);
+}
+
+// The kernel compiled for two CTAs of 512 threads on an SM (56 to 64 registers) or for
+// three (40).  Three pay where the grid is more than four and a half CTAs per SM and most
+// of a CTA's threads have work: 46x26 vs 97x12 with 90 planes 462 -> 356 us, 32x30 vs
+// 92x18, 68: 366 -> 304, 44x27 vs 41x41, 82: 353 -> 295 (with a 4-byte box per row and
+// about 40 registers they took 359, 315 and 286).  On smaller grids the narrower register
+// set costs: 17x63 vs 24x31, 42 (408 CTAs): 93 -> 110.
+template <int K>
+cudaError_t launch_cols(const ColPlan& c, const float* g, int np, int ha, int wa, int hb, int wb, const long long* t,
+                        int64_t stride, float* c_hi, float* c_lo, cudaStream_t st) {
+    const int64_t ctas = (int64_t)hb * ((ha + K - 1) / K);
+    if (c.threads == 512 && c.smem <= kR4SmemCap / 3 && ctas > 700 && c.G * wa >= 360)
+        return launch_cols_t<K, 3>(c, g, np, ha, wa, hb, wb, t, stride, c_hi, c_lo, st);
+    return launch_cols_t<K, 1>(c, g, np, ha, wa, hb, wb, t, stride, c_hi, c_lo, st);
 }
 }  // namespace
 
