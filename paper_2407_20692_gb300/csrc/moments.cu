@@ -24,9 +24,10 @@
 // Each (frame chunk, 128 x 256 output tile) of a problem is one work unit; its
 // exact partial sum goes to its own slot of the workspace, and the fold step
 // adds the slots into int64.  (Finishing Eq. (1) in this epilogue was measured
-// slower on GB300: the correctly rounded quotients keep the epilogue warps from
-// draining the next tile's segments, and the MMAs wait; the fold kernel spreads
-// that work over every SM instead.)  Integer addition is associative, so the
+// slower on GB300, with a quotient of about 100 instructions: it kept the epilogue
+// warps from draining the next tile's segments, and the MMAs waited; the fold kernel
+// spreads that work over every SM instead.  Not measured with the present quotient of
+// about 40.)  Integer addition is associative, so the
 // split over chunks, segments and CTAs never changes the result.  One launch
 // serves one problem (a correlation) or up to kMaxGroup problems of uneven
 // shapes (a batch): the persistent CTAs walk one list of units, each unit naming
@@ -34,13 +35,15 @@
 //
 // Persistent, warp-specialised CTA (one per SM, 320 threads):
 //   warp 0   : TMA producer (128-byte swizzled tiles, 4-deep ring)
-//   warp 1   : tensor-memory allocator and single-thread MMA issuer
+//   warp 1   : tensor-memory allocator and MMA issuer (the whole warp runs the loop,
+//              one lane issues)
 //   warps 2-9: epilogue, tensor memory -> registers -> global (TMEM lanes 32*(w%4)..)
-// Two TMEM accumulators let the epilogue of one unit (binary frames) or one
-// exact FP32 segment (8-bit frames) overlap the MMAs of the next; the 8-bit
-// int32 running sums of a unit stay in the epilogue threads' registers.  Every barrier wait is bounded; on a
-// time-out the CTA records the error, drains its own copies and MMAs, frees its
-// tensor memory and returns.
+// Two TMEM accumulators let the epilogue of one exact FP32 segment (8-bit frames) or
+// one unit (binary frames, tiles of 128 columns) overlap the MMAs of the next; binary
+// tiles of 256 columns have one, which their epilogue empties into registers first.
+// The 8-bit int32 running sums of a unit stay in the epilogue threads' registers.
+// Every barrier wait is bounded; on a time-out the CTA records the error, drains its
+// own copies and MMAs, frees its tensor memory and returns.
 #include "kernels.cuh"
 #include "ptx.cuh"
 

@@ -146,8 +146,7 @@ __global__ void __launch_bounds__(256) refocus_xtables_kernel(const PlaneBlock p
 // serves PB planes while each thread keeps the sums of all of them.
 template <int WS, int KR, int PT>
 __global__ void __launch_bounds__(kBandThreads, 1) refocus_band_kernel(const __grid_constant__ CUtensorMap tm,
-                                                                           const BandGeom g, const PlaneBlock pl,
-                                                                           float* __restrict__ ubuf) {
+                                                                           const BandGeom g, float* __restrict__ ubuf) {
     constexpr int NW = kBandThreads / 32;
     constexpr int PB = PT;
     static_assert(PT % 2 == 0, "planes are processed in pairs");
@@ -755,27 +754,27 @@ cudaError_t set_smem_attr(K kernel, int slot, size_t bytes) {
 }
 
 template <int WS, int KR, int PT>
-cudaError_t launch_band_t(const CUtensorMap* tm, const BandGeom& g, const PlaneBlock& pl, float* ubuf, size_t smem,
+cudaError_t launch_band_t(const CUtensorMap* tm, const BandGeom& g, float* ubuf, size_t smem,
                           int grid, cudaStream_t st, int slot) {
     auto kern = refocus_band_kernel<WS, KR, PT>;
     cudaError_t e = set_smem_attr(kern, slot, kSmemCap);
     if (e != cudaSuccess) return e;
-    return launch_kernel(true, kern, grid, kBandThreads, smem, st, *tm, g, pl, ubuf);
+    return launch_kernel(true, kern, grid, kBandThreads, smem, st, *tm, g, ubuf);
 }
 
-cudaError_t launch_band(const BandPlan& b, const CUtensorMap* tm, const BandGeom& g, const PlaneBlock& pl,
+cudaError_t launch_band(const BandPlan& b, const CUtensorMap* tm, const BandGeom& g,
                         float* ubuf, int grid, cudaStream_t st) {
-    if (b.KR == 2) return launch_band_t<40, 2, 8>(tm, g, pl, ubuf, b.smem, grid, st, 0);
+    if (b.KR == 2) return launch_band_t<40, 2, 8>(tm, g, ubuf, b.smem, grid, st, 0);
     switch (b.WS) {
-        case 40: return launch_band_t<40, 8, 4>(tm, g, pl, ubuf, b.smem, grid, st, 1);
-        case 72: return launch_band_t<72, 8, 4>(tm, g, pl, ubuf, b.smem, grid, st, 2);
-        case 104: return launch_band_t<104, 8, 4>(tm, g, pl, ubuf, b.smem, grid, st, 3);
-        case 136: return launch_band_t<136, 8, 4>(tm, g, pl, ubuf, b.smem, grid, st, 4);
-        case 200: return launch_band_t<200, 8, 4>(tm, g, pl, ubuf, b.smem, grid, st, 5);
-        case 256: return launch_band_t<256, 8, 4>(tm, g, pl, ubuf, b.smem, grid, st, 6);
-        case 288: return launch_band_t<288, 8, 4>(tm, g, pl, ubuf, b.smem, grid, st, 7);
-        case 416: return launch_band_t<416, 8, 4>(tm, g, pl, ubuf, b.smem, grid, st, 8);
-        case 544: return launch_band_t<544, 8, 4>(tm, g, pl, ubuf, b.smem, grid, st, 9);
+        case 40: return launch_band_t<40, 8, 4>(tm, g, ubuf, b.smem, grid, st, 1);
+        case 72: return launch_band_t<72, 8, 4>(tm, g, ubuf, b.smem, grid, st, 2);
+        case 104: return launch_band_t<104, 8, 4>(tm, g, ubuf, b.smem, grid, st, 3);
+        case 136: return launch_band_t<136, 8, 4>(tm, g, ubuf, b.smem, grid, st, 4);
+        case 200: return launch_band_t<200, 8, 4>(tm, g, ubuf, b.smem, grid, st, 5);
+        case 256: return launch_band_t<256, 8, 4>(tm, g, ubuf, b.smem, grid, st, 6);
+        case 288: return launch_band_t<288, 8, 4>(tm, g, ubuf, b.smem, grid, st, 7);
+        case 416: return launch_band_t<416, 8, 4>(tm, g, ubuf, b.smem, grid, st, 8);
+        case 544: return launch_band_t<544, 8, 4>(tm, g, ubuf, b.smem, grid, st, 9);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1018,7 +1017,7 @@ cudaError_t refocus_run(const float* gamma_f32, int ha, int wa, int hb, int wb, 
             g.timeout_ns = timeout_ns;
             const int64_t units = (int64_t)hb * g.n_pb * g.n_bands;
             const int grid = units < sm_count ? (int)units : sm_count;
-            e = launch_band(b, &tm, g, pb, ubuf, grid, st);
+            e = launch_band(b, &tm, g, ubuf, grid, st);
         }
         if (e != cudaSuccess) return e;
         YGeom y{ha, wa, hb, RB, p0};
