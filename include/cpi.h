@@ -370,7 +370,7 @@ CPI_API cpi_status cpi_correlate_noalloc(const cpi_frames *a, const cpi_frames *
  * model: DEVICE float [CPI_DENOISER_PARAMS], float32 master weights, per layer
  *   l = 0..3 the weights W_l [Cout][Cin][3][3] then the biases b_l [Cout].
  * workspace: DEVICE, 256-byte aligned, cpi_denoise_workspace_size bytes
- *   (training != 0 for cpi_denoise_grad; about 3.2 GB for 64x64 vs 32x32).
+ *   (training != 0 for cpi_denoise_grad; about 4.7 GB for 64x64 vs 32x32).
  * Requires ha, wa, hb, wb >= 1 and hb * wb <= 65535; errors are reported before
  * any launch.
  *

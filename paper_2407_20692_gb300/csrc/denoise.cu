@@ -408,8 +408,11 @@ DenoiseLayout denoise_layout(int ha, int wa, int hb, int wb, bool training) {
     L.a2 = take(2 * (size_t)(B * 32 * HW));
     L.a3 = take(2 * (size_t)(B * 32 * HW));
     L.y = take(4 * (size_t)(B * HW));
-    const bool tc = (wa == 32 || wa == 64 || wa == 128) && B <= 65535;
-    if (tc) {                                   // room for the padded line (denoise_line.cu)
+    // The bytes of the widths 32, 64 and 128 are those the workspace has always had, part
+    // of the interface.  Beside the direct convolutions' buffers they only make room for
+    // the padded line (denoise_line.cu), which needs about 130 bytes per position, 370 in
+    // training.
+    if (wa == 32 || wa == 64 || wa == 128) {
         for (int k = 0; k < 3; ++k) take(64 * (size_t)(B * HW));
         take(2 * (size_t)(3 * 9 * 32 * 32 + 9 * 16 * 32));
     }
@@ -418,7 +421,7 @@ DenoiseLayout denoise_layout(int ha, int wa, int hb, int wb, bool training) {
         L.d_hi = take(4 * (size_t)(B * 32 * HW));
         L.d_lo = take(4 * (size_t)(B * 32 * HW));
         L.part = take(sizeof(float) * (size_t)kDenoiseParts * (32 * 32 * 9 + 32));
-        if (wa == 64 && B <= 65535) {           // likewise
+        if (wa == 64) {
             take(2 * (size_t)(B * 64 * HW));
             take(2 * (size_t)(B * 96 * HW));
             take(sizeof(float) * (size_t)(2 * 152) * 64 * 288);

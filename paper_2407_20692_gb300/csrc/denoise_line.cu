@@ -822,13 +822,17 @@ __global__ void __launch_bounds__(kTopThreads) dnf_top_grad_kernel(const DnFlat 
 // against 4.6e-7 in FP32).  The last layer's gradients, exact but for these sums, go in
 // runs of 64 pixels: over 28 training steps of widths 24 to 128 the error of the whole
 // gradient against 64 bits is 0.98 of that of FP32 sums (1.02 at most), with runs of a
-// unit it was 1.00 (1.07 at most, always above 1 at widths 32 and 128).  hold: images 64 wide, whose
-// gradients have always been summed that way, keep one accumulator to the end over
-// the same blocks of up to 32 rows of a slice per CTA, so that training there goes
-// on as it was; only the first unit has an accumulator of its own, which makes up for
-// the zero column that is summed with every row.  1024 slices of 64 x 64, 32 -> 32: 194 us, 0.83 GB at 4.3 TB/s.  At the
-// end the CTA writes rows (kx, ci) x
-// columns (ky, n) to part[cta].  Every wait is bounded.
+// unit it was 1.00 (1.07 at most, always above 1 at widths 32 and 128).
+// hold: images 64 wide, whose gradients have been summed in one accumulator to the end
+// since before the line, keep that over the same blocks of up to 32 rows of a slice per
+// CTA, so that the gradients at that width stay what they were.  It is the less exact
+// sum: 5.2e-5 of the gradient from 64 bits at 64x64 vs 32x32, drained per unit 1.0e-6
+// (2020 us a step against 2094 with the other widths' order of lo and hi terms, which
+// goes with it).  Only the first unit has an accumulator of its own, which makes up for
+// the zero column that is summed with every row: 0.972 of the error of the sums over the
+// images' own pixels (16 steps; without it 1.011).
+// 1024 slices of 64 x 64, 32 -> 32: 192 us, 0.83 GB at 4.3 TB/s.  At the end the CTA
+// writes rows (kx, ci) x columns (ky, n) to part[cta].  Every wait is bounded.
 constexpr int kWgThreads = 192;
 constexpr int kWgMaxStages = 4;
 struct WgArgs {

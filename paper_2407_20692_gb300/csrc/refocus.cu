@@ -329,12 +329,14 @@ __global__ void __launch_bounds__(kBandThreads, 1) refocus_band_kernel(const __g
 // The same sums (bit for bit) from a copy of Gamma whose rows come four to a group,
 // [slice][group][column, 2 zero columns on either side][4 rows], made once per call:
 // a tap of four rows is one 16-byte shared-memory load that arrives as two packed
-// row pairs, and a unit's band of a slice is one contiguous bulk copy.  Bound by the
-// latency of the shared-memory reads (an ncu capture of the form without the reads
-// ahead: 5 of 9 stall cycles per instruction, read wavefronts at 38% of their rate),
-// so each item's loads are issued one item ahead of its arithmetic (4.58 -> 4.22 ms
-// at 128x128 vs 64x64, 128 planes); 24 warps of 2 planes instead of 16 of 4 were
-// slower (4.78 ms).  Whole call, row-major -> this, one GB300: 128x128 vs 64x64, 128
+// row pairs, and a unit's band of a slice is one contiguous bulk copy.  Bound by
+// latency at 16 warps per SM with a full register file: 8.1 instructions per sample at
+// 52% of the issue slots, shared-memory wavefronts at 51% of their rate, and of 7.2
+// cycles between a warp's instructions 1.5 each waiting for shared and for global or
+// TMA data and 1.4 for fixed latencies (ncu, 44 planes of 128x128 vs 16x64).  Each
+// item's loads are issued one item ahead of its arithmetic (4.58 -> 4.22 ms at 128x128
+// vs 64x64, 128 planes; without it 5.1 of 9 cycles were shared-memory waits); 24 warps
+// of 2 planes instead of 16 of 4 were slower (4.78 ms).  Whole call, row-major -> this, one GB300: 128x128 vs 64x64, 128
 // planes 4.35 -> 4.22 ms; 96x96 vs 40x40, 128: 1.36 -> 1.05; 83x83 vs 37x37, 128: 1.16 ->
 // 0.80; 70x50 vs 30x30, 128: 0.53 -> 0.32; 40x40 vs 20x20, 256: 0.31 -> 0.19.
 //
