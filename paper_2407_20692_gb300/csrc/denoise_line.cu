@@ -1128,15 +1128,17 @@ __global__ void __launch_bounds__(256) dnf_wgrad_reduce_kernel(const float* __re
 }
 
 // ------------------------------------------------------------------ host
-// Short lines at the tensor-core widths gain from kernels placed ahead, on long ones the
-// gaps do not count and the placed CTAs cost.  Chained and plain, us: 32x64 vs 8x9 (154
+// Short lines gain from kernels placed ahead, on long ones the gaps do not count and the
+// placed CTAs cost.  Chained and plain at the tensor-core widths, us: 32x64 vs 8x9 (154
 // thousand positions) 56 / 62, 64x64 vs 14x16 (946 thousand) 169 / 171, 32x32 vs 31x32
 // (1.08 million) 180 / 182, 64x64 vs 20x20 (1.69 million) 253 / 248, 64x64 vs 32x32 547 /
-// 517; training 182 / 209, 569 / 587, 632 / 651, 922 / 936, 2052 / 2029.  The FP32
-// kernels fill an SM's registers, so whatever is placed ahead takes a CTA's place: 24x31
-// vs 8x8 136 / 117, 47x53 vs 10x12 421 / 377, 83x83 vs 20x20 2591 / 2482 (training 3858 /
-// 3706).
-bool in_chain(const DnFlat& g) { return g.tensor && g.Q < (1u << 20); }
+// 517; training 182 / 209, 569 / 587, 632 / 651, 922 / 936, 2052 / 2029.  The FP32 layers of
+// the other widths are launched plainly on any line; two of their CTAs fill an SM.  With
+// them chained and not (the rest of the call chained): 24x31 vs 8x8 135 / 117, 30x25 vs
+// 9x8 163 / 117, 47x53 vs 10x12 420 / 372, 60x87 vs 12x12 746 / 709, 83x83 vs 12x12 1020 /
+// 975, the other way round 94x60 vs 8x8 429 / 441 and 43x58 vs 10x14 426 / 438; training
+// 221 / 204, 251 / 207, 617 / 567, 1122 / 1071, 1511 / 1459, 643 / 654, 636 / 646.
+bool in_chain(const DnFlat& g) { return g.Q < (1u << 20); }
 
 template <typename K>
 cudaError_t allow_smem(K kernel, bool (&done)[64]) {
@@ -1205,7 +1207,7 @@ cudaError_t launch_forward(DnFlat g, const ConvArgs& a, const float* w, int sm_c
     int grid = (MODE == kTrain ? 1 : 2) * sm_count;
     if (g.n_units < grid) grid = g.n_units;
     if (ctas) *ctas = grid;
-    return launch_kernel(in_chain(g), dnf_conv_exact_kernel<CIN, COUT, MODE>, grid, kExThreads, smem, st, g, a, w);
+    return launch_kernel(false, dnf_conv_exact_kernel<CIN, COUT, MODE>, grid, kExThreads, smem, st, g, a, w);
 }
 
 template <int CIN, int KC, int COUT, int kRun = 0>
