@@ -571,7 +571,7 @@ def rooflines(ma, mb, n, n_planes, bits, ms, workload):
     smem = n_planes * ma * mb * 8.0
     smem_peak = SM_COUNT * SMEM_BYTES_PER_CLK * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e9
     a = smem / (ms["refocus"] / 1e3) / 1e9
-    out["refocus"] = {"kernel": "refocus (row-band x stage, 4 planes per staged slice band, + y stage over angular rows)",
+    out["refocus"] = {"kernel": "refocus (x stage on row bands, row-major or interleaved, 4 planes per staged slice band, + y stage over angular rows)",
                       "bound": "hbm", "achieved": eff, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                       "frac": eff / peaks["hbm_gbs"], "traffic": _traffic("refocus", workload),
                       "peak_source": f"{src} hbm copy", "ms": ms["refocus"],
